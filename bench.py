@@ -210,10 +210,8 @@ class Ensembles:
         self.rosen.rosen_reduce(it["rin"], it["stats"], self.ws, stream)
 
     def launches_per_step(self):
-        # Growth and two reduction kernels per ensemble; hard spheres grow in
-        # two passes (growth, then the deferred chains).
-        return sum(4 if it["kind"] == "offlattice" and REAL_POT == "hard_sphere" else 3
-                   for it in self.items)
+        # Growth and two reduction kernels per ensemble.
+        return 3 * len(self.items)
 
 
 def run_ours(args):
@@ -306,7 +304,7 @@ def run_ours(args):
             sops = brute_offlattice_ops(N, K_TRIALS) * C
             part.update({"fp64_redecided_steps": cnt[0] / reps,
                          "listed_beads_per_step": listed / (C * (N - 1))})
-            kname = ("offlattice_queue_kernel<16,2,hard sphere,defer> + offlattice_deferred_kernel"
+            kname = ("offlattice_wide_kernel<4,8>"
                      if REAL_POT == "hard_sphere"
                      else "offlattice_queue_kernel<LJ, k=%d, beta eps %g>" % (K_TRIALS, REAL_BETA))
         part["ops_per_chain"] = ops / C

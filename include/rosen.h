@@ -232,12 +232,10 @@ typedef struct rosen_offlattice_out {
  * distance lies within about 1e-13 N of sigma^2 or of cutoff^2, or the
  * selection draw within a relative 1e-13 N of a prefix-sum boundary (the
  * tests require >= 99.9% equal paths; all tested chains take them).
- * Scratch: the call takes 8 bytes (plus, for hard spheres with N <= 128, a
- * bit per chain) from the device's stream-ordered allocator on `stream` and
- * frees it there: a chain counter for the persistent grid and the mask of
- * chains deferred to the FP64 second pass.  If that allocation fails, the
- * chains grow in one pass with one block per few chains; the results are
- * the same bit for bit.
+ * Scratch: the call takes 16 bytes from the device's stream-ordered allocator
+ * on `stream` and frees them there: a chain counter for the persistent grid.
+ * If that allocation fails, every chain group grows one chain; the results
+ * are the same bit for bit.
  * Errors: EINVAL for N outside [2, 1024], k outside [1, 128], bad chain
  * range, unknown potential, sigma/cutoff/beta_eps out of range, unknown
  * flags or lanes_per_chain, max_attempts outside [0, ROSEN_MAX_ATTEMPTS].

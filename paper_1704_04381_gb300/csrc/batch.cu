@@ -47,7 +47,7 @@ struct ClassPlan {
     bool lattice;
     bool lj;
     std::vector<char> own;      // per member: grown by its own single-ensemble launch
-    std::vector<size_t> own_off;   // real space: offset of its counters and mask in d_own
+    std::vector<size_t> own_off;   // real space: offset of its chain counter in d_own
     void *d_own = nullptr;      // real space: scratch of the members with their own launch
     size_t own_bytes = 0;
     bool longc = false; // long chains: members grown one after another by the
@@ -248,8 +248,6 @@ int upload_items(ClassPlan &c, const std::vector<BatchItem> &items)
 // range launches (default lanes per chain, as rosen_*_grow would grow them).
 int launch_own(const rosen_batch *b, const ClassPlan &c, cudaStream_t s)
 {
-    if (c.d_own && cudaMemsetAsync(c.d_own, 0, c.own_bytes, s) != cudaSuccess)
-        return set_error(ROSEN_ECUDA, "batch: clearing the members' scratch");
     for (size_t m = 0; m < c.members.size(); ++m) {
         if (!c.own[m]) continue;
         const int e = c.members[m];
@@ -260,10 +258,7 @@ int launch_own(const rosen_batch *b, const ClassPlan &c, cudaStream_t s)
         } else {
             const rosen_offlattice_params p = off_params(b->ens[e], 0);
             unsigned char *sc = static_cast<unsigned char *>(c.d_own) + c.own_off[m];
-            st = offlattice_grow_range(&p, &b->off_out[e], 0, p.C, sc,
-                                       reinterpret_cast<uint32_t *>(
-                                           sc + offlattice_range_counter_bytes()),
-                                       s);
+            st = offlattice_grow_range(&p, &b->off_out[e], 0, p.C, sc, s);
         }
         if (st != ROSEN_OK) return st;
     }
@@ -595,7 +590,7 @@ int create(rosen_batch *b, const rosen_ensemble *ens, int n)
             continue;
         }
         // Members that fill the GPU by themselves get their own launch
-        // (real space: with their own chain counters and deferral mask).
+        // (real space: with their own chain counters).
         c.own.assign(c.members.size(), 0);
         c.own_off.assign(c.members.size(), 0);
         for (size_t m = 0; m < c.members.size(); ++m) {
@@ -612,8 +607,7 @@ int create(rosen_batch *b, const rosen_ensemble *ens, int n)
                 c.own[m] = 1;
                 if (!c.lattice) {
                     c.own_off[m] = c.own_bytes;
-                    c.own_bytes += align256(offlattice_range_counter_bytes() +
-                                            offlattice_range_mask_bytes(x.C));
+                    c.own_bytes += align256(offlattice_range_counter_bytes());
                 }
             }
         }

@@ -31,19 +31,13 @@ void offlattice_make_args(const rosen_offlattice_params *p, const rosen_offlatti
                           unsigned long long *counters, void *out);
 int offlattice_default_lanes(int k, bool lj, int N = 0);
 // Local chains [c_lo, c_hi) of a validated ensemble (shared-memory kernels,
-// N <= 1024), with caller-owned scratch: counters of
+// N <= 1024), with a caller-owned chain counter of
 // offlattice_range_counter_bytes() (16-byte aligned, zeroed by the call; one
-// set per range that may run concurrently with another) and the deferral
-// mask of offlattice_range_mask_bytes(C) bytes (4-byte aligned, zero before
-// the first range of the ensemble, shared by all its ranges).  For hard
-// spheres, ranges that run at the same time must not share mask words: start
-// them at multiples of 32 chains.  Outputs are those of
+// per range that may run concurrently with another).  Outputs are those of
 // rosen_offlattice_grow, bit for bit.
 size_t offlattice_range_counter_bytes();
-size_t offlattice_range_mask_bytes(int64_t C);
 int offlattice_grow_range(const rosen_offlattice_params *p, const rosen_offlattice_out *o,
-                          int64_t c_lo, int64_t c_hi, void *counters, uint32_t *mask,
-                          cudaStream_t s);
+                          int64_t c_lo, int64_t c_hi, void *counter, cudaStream_t s);
 // Chains the GPU grows at the same time for this ensemble (0 on error).
 int64_t offlattice_resident_chains(const rosen_offlattice_params *p);
 int offlattice_batch_prepare(int G, int T, bool lj, int Nmax, int *chains_per_block, size_t *smem,

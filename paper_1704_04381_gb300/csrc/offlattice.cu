@@ -26,14 +26,18 @@
 //
 // Scheduling: the grid is what the GPU holds at once, and every group takes
 // its next chain from a counter (chains differ in cost by their re-decisions
-// and dead ends).  Short hard-sphere chains grow in two passes, the second
-// regrowing, with the FP64 path, the few chains the first could not decide.
+// and dead ends).  Lennard-Jones chains, and both potentials in a batch, grow
+// with the kernels below; hard spheres grow with those of offlattice_wide.cuh,
+// which takes the same steps with fewer lanes per chain.
 #include <math.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "internal.cuh"
 #include "offlattice_chain.cuh"
+#include "offlattice_wide.cuh"
 
 namespace rosen {
 namespace {
@@ -61,7 +65,7 @@ __global__ void __launch_bounds__(256, 4) offlattice_group_kernel(const OffArgs 
 // block holds no lanes idle while its slowest chain finishes (chains differ
 // in their number of FP64 re-decisions and dead ends).  The grid is what the
 // GPU holds at once.
-template <int G, int T, bool LJ, bool kDefer = false>
+template <int G, int T, bool LJ>
 __global__ void __launch_bounds__(256, 4) offlattice_queue_kernel(const OffArgs a,
                                                                   int chains_per_block,
                                                                   unsigned long long *next,
@@ -81,51 +85,7 @@ __global__ void __launch_bounds__(256, 4) offlattice_queue_kernel(const OffArgs 
         if (g.gl == 0) c = (unsigned long long)c_lo + atomicAdd(next, 1ull);
         c = g.bcast(c, 0);
         if (c >= (unsigned long long)c_hi) break;
-        off_chain<G, T, LJ, ChainSmem, kDefer>(a, (int64_t)c, w, g, logm);
-    }
-}
-
-// Second pass of two-pass growth: the chains of [c_lo, c_hi) whose bits the
-// first pass set, grown again from the start with the FP64 re-decision
-// compiled in.  Warps take 32-chain words of the bit mask from a counter, so
-// the few deferred chains spread evenly; the groups of a warp take a word's
-// set bits together, one each per round, so they step in lock-step as in
-// the first pass instead of diverging.
-template <int G, int T, bool LJ>
-__global__ void __launch_bounds__(256, 4) offlattice_deferred_kernel(const OffArgs a,
-                                                                     int chains_per_block,
-                                                                     unsigned int *next,
-                                                                     int64_t c_lo, int64_t c_hi)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float *logm = reinterpret_cast<float *>(smem_raw);
-    fill_log_table(logm);
-    __syncthreads();
-
-    const Group<G> g;
-    const int cib = threadIdx.x / G;
-    const ChainSmem w = carve(smem_raw + kTable * sizeof(float) +
-                                  (size_t)cib * chain_smem_bytes(a.N, LJ), a.N, LJ);
-    const int64_t w_lo = c_lo / 32, w_hi = (c_hi + 31) / 32;
-    const int gw = (threadIdx.x & 31) / G;     // this group's place in its warp
-    for (;;) {
-        int64_t q = 0;
-        if ((threadIdx.x & 31) == 0) q = w_lo + (int64_t)atomicAdd(next, 1u);
-        q = __shfl_sync(0xffffffffu, q, 0);
-        if (q >= w_hi) break;
-        // Only the chains of this range (the words at its ends may hold
-        // chains of neighbouring ranges).
-        const int64_t b0 = q * 32;
-        uint32_t m = a.deferred[q];
-        if (b0 < c_lo) m &= ~0u << (uint32_t)(c_lo - b0);
-        if (b0 + 32 > c_hi) m &= (c_hi - b0 >= 32) ? ~0u : ((1u << (uint32_t)(c_hi - b0)) - 1u);
-        while (m) {
-            uint32_t mine = m;                   // the gw-th set bit of m, if any
-            for (int t = 0; t < gw && mine; ++t) mine &= mine - 1u;
-            if (mine) off_chain<G, T, LJ>(a, b0 + __ffs(mine) - 1, w, g, logm);
-            for (int t = 0; t < 32 / G && m; ++t) m &= m - 1u;
-            __syncwarp();
-        }
+        off_chain<G, T, LJ>(a, (int64_t)c, w, g, logm);
     }
 }
 
@@ -171,7 +131,7 @@ __global__ void __launch_bounds__(256, 4) offlattice_batch_kernel(const OffArgs 
             __syncwarp(g.mask);
             cur = (int)bi.ens;
         }
-        off_chain<G, T, LJ, ChainSmem, false, true>(my, bi.c0 + off, w, g, logm);
+        off_chain<G, T, LJ, ChainSmem, true>(my, bi.c0 + off, w, g, logm);
     }
 }
 
@@ -212,161 +172,166 @@ int chains_per_block_for(int G, int N, bool lj)
     return chains;
 }
 
-// Scratch of a range launch: 16 bytes of counters (the chain counter, 8
-// bytes, and the second pass's word counter, 4 bytes), zeroed by every
-// launch, and the deferral mask, one bit per chain of the ensemble, which
-// must be zero before the first launch over an ensemble's chains.  Launches
-// that may run at the same time need counters of their own; they can share
-// the mask (their chain ranges are disjoint).
+// Scratch of a range launch: the chain counter, zeroed by every launch.
+// Launches that may run at the same time need counters of their own.
 constexpr size_t kScratchHeader = 16;
 
-size_t mask_bytes(int64_t C) { return (size_t)((C + 31) / 32) * sizeof(uint32_t); }
-
-// Growth of local chains [c_lo, c_hi).  Groups take chains from a counter
-// (offlattice_queue_kernel); the grid is what the GPU holds at once.  Short
-// hard-sphere chains (N <= 128) grow in two passes: their FP32 decisions are
-// almost never ambiguous (about 2% of N = 64, k = 32 chains meet one such
-// step), but the FP64 re-decision path, compiled into the growth kernel,
-// costs every chain registers and time (the kernel without it runs 11%
-// faster).  So the first pass has no FP64 path and defers the chains that
-// need it; the second regrows only those, with it.  Longer chains meet
-// ambiguous steps more often (a third of N = 512 chains), and regrowing them
-// costs more than the first pass saves, so they grow in one pass.  Every
-// chain's outputs are those of the one-pass kernel, bit for bit.
-template <int G, int T, bool LJ>
-int launch_range(const OffArgs &a, int N, int64_t c_lo, int64_t c_hi, void *counters,
-                 uint32_t *mask, cudaStream_t s)
+int set_cuda_error(cudaError_t e)
 {
-    const int chains = chains_per_block_for(G, N, LJ);
-    const size_t smem = kTable * sizeof(float) + (size_t)chains * chain_smem_bytes(N, LJ);
+    return set_error(ROSEN_ECUDA, "rosen_offlattice_grow: %s", cudaGetErrorString(e));
+}
+
+// ---- Lennard-Jones: a group of G lanes per chain -----------------------------------
+// Local chains [c_lo, c_hi): groups take them from the counter, the grid is
+// what the GPU holds at once.  Without a counter, one block per
+// chains_per_block chains (the same outputs).
+template <int G, int T>
+int launch_lj(const OffArgs &a, int64_t c_lo, int64_t c_hi, void *counter, cudaStream_t s,
+              int64_t *resident)
+{
+    const int chains = chains_per_block_for(G, a.N, true);
+    const size_t smem = kTable * sizeof(float) + (size_t)chains * chain_smem_bytes(a.N, true);
     const int threads = chains * G;
-    const int64_t n = c_hi - c_lo;
-    const int64_t blocks = (n + chains - 1) / chains;
-    const bool two_pass = !LJ && N <= 128;
-    unsigned char *sc = static_cast<unsigned char *>(counters);
-    unsigned long long *next = reinterpret_cast<unsigned long long *>(sc);
-    unsigned int *wnext = reinterpret_cast<unsigned int *>(sc + 8);
-    OffArgs d = a;
-    if (two_pass) d.deferred = mask;
-    cudaError_t e = cudaMemsetAsync(sc, 0, kScratchHeader, s);
+    const int64_t blocks = (c_hi - c_lo + chains - 1) / chains;
+    if (!counter && !resident) {
+        allow_max_smem(offlattice_group_kernel<G, T, true>);
+        offlattice_group_kernel<G, T, true><<<(unsigned)blocks, threads, smem, s>>>(a, chains);
+        return check_launch("rosen_offlattice_grow");
+    }
     int dev = 0, sms = 0, bps = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // The first pass without the FP64 path, or the one pass with it.
-    auto first = two_pass ? offlattice_queue_kernel<G, T, LJ, !LJ>
-                          : offlattice_queue_kernel<G, T, LJ, false>;
-    if (e == cudaSuccess) e = allow_max_smem(first);
+    if (e == cudaSuccess) e = allow_max_smem(offlattice_queue_kernel<G, T, true>);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, first, threads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, offlattice_queue_kernel<G, T, true>,
+                                                          threads, smem);
+    if (resident) {
+        *resident = e == cudaSuccess ? (int64_t)bps * sms * chains : 0;
+        if (e != cudaSuccess) cudaGetLastError();
+        return ROSEN_OK;
+    }
+    if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, kScratchHeader, s);
     if (e == cudaSuccess) {
         int64_t grid = (int64_t)(bps > 0 ? bps : 1) * sms;
         if (grid > blocks) grid = blocks;
-        first<<<(unsigned)grid, threads, smem, s>>>(d, chains, next, c_lo, c_hi);
-        if constexpr (!LJ) {
-            if (two_pass) {
-                int bps2 = 0;
-                e = allow_max_smem(offlattice_deferred_kernel<G, T, LJ>);
-                if (e == cudaSuccess)
-                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                        &bps2, offlattice_deferred_kernel<G, T, LJ>, threads, smem);
-                const int64_t words = (c_hi + 31) / 32 - c_lo / 32;
-                int64_t grid2 = (int64_t)(bps2 > 0 ? bps2 : 1) * sms;
-                if (grid2 > (words + chains - 1) / chains) grid2 = (words + chains - 1) / chains;
-                if (e == cudaSuccess)
-                    offlattice_deferred_kernel<G, T, LJ>
-                        <<<(unsigned)grid2, threads, smem, s>>>(d, chains, wnext, c_lo, c_hi);
-            }
+        offlattice_queue_kernel<G, T, true><<<(unsigned)grid, threads, smem, s>>>(
+            a, chains, static_cast<unsigned long long *>(counter), c_lo, c_hi);
+        e = cudaGetLastError();
+    }
+    return e == cudaSuccess ? ROSEN_OK : set_cuda_error(e);
+}
+
+// ---- hard spheres: the wide kernel ---------------------------------------------------
+using WideFn = void (*)(const OffArgs, const WideShape, unsigned long long *, int64_t, int64_t);
+
+struct WidePlan {
+    WideFn fn;
+    int G, warps;        // lanes per chain, warps per block
+    size_t smem;
+    WideShape sh;
+};
+
+// Shape for n chains of N beads and k trials whose sums follow gref lanes per
+// chain.  G is the fewest lanes that hold k trials (8 each) and whose scan bits
+// fit a word (N <= 32 G); with few chains it doubles while the warps stay
+// within 9 per SM, where the lanes would idle otherwise and a step's latency
+// counts (N = 64, k = 32, G = 4 / 8 / 16: 2500 chains 0.192 / 0.172 / 0.162
+// ms, 5000 0.210 / 0.186 / 0.243, 10^4 0.264 / 0.270 / 0.342).  A block has
+// the warps that fill an SM's shared memory best, at most 16 (128 registers a
+// thread), fewer where there are not enough chains for every SM.
+WidePlan wide_plan(const OffArgs &a, int gref, int64_t n, int sms)
+{
+    WidePlan w;
+    const int N = a.N, k = a.k;
+    int G = 4;
+    while (8 * G < k || 32 * G < N) G *= 2;
+    while (G < 32 && n * 2 * G <= (int64_t)32 * 9 * sms) G *= 2;
+    const int T = ((k + G - 1) / G + 1) / 2 * 2;
+    w.fn = nullptr;
+#define ROSEN_WIDE(GG, TT) if (G == GG && T == TT) w.fn = offlattice_wide_kernel<GG, TT>;
+    ROSEN_WIDE(4, 2) ROSEN_WIDE(4, 4) ROSEN_WIDE(4, 6) ROSEN_WIDE(4, 8)
+    ROSEN_WIDE(8, 2) ROSEN_WIDE(8, 4) ROSEN_WIDE(8, 6) ROSEN_WIDE(8, 8)
+    ROSEN_WIDE(16, 2) ROSEN_WIDE(16, 4) ROSEN_WIDE(16, 6) ROSEN_WIDE(16, 8)
+    ROSEN_WIDE(32, 2) ROSEN_WIDE(32, 4)
+#undef ROSEN_WIDE
+    w.G = G;
+    w.sh.np = wide_np(N, G);
+    w.sh.stride = wide_stride(N, G);
+    w.sh.gref = gref;
+    // |g|^2 from the hi words alone differs from the float-float value by the
+    // lo words (<= 6e-8 N per axis) and FP32 rounding (as in
+    // rosen_offlattice_grow_long); doubled.
+    const double rf2 = a.rf2, rf = sqrt(rf2), d = 6e-8 * N + 1e-6;
+    w.sh.pre2 = (float)(rf2 + 2.0 * (3.5 * (rf + 1.0) * d + 3.0 * d * d + 4e-6 * rf2) + 1e-6);
+    const size_t head = kTable * sizeof(float) + kWideSelBytes;
+    const size_t per_warp = (size_t)(32 / G) * w.sh.stride * sizeof(float);
+    const size_t sm = (size_t)max_dynamic_smem() + 1024;     // (1 KB per block is reserved)
+    int best = 0;
+    w.warps = 1;
+    for (int q = 1; q <= 16; ++q) {
+        const int held = std::min((int)(sm / (head + q * per_warp + 1024)), 16 / q) * q;
+        if (held > best) {
+            best = held;
+            w.warps = q;
         }
-        if (e == cudaSuccess) e = cudaGetLastError();
     }
-    if (e != cudaSuccess)
-        return set_error(ROSEN_ECUDA, "rosen_offlattice_grow: %s", cudaGetErrorString(e));
-    return ROSEN_OK;
+    const int64_t warps = (n * G + 31) / 32;
+    if (warps < (int64_t)w.warps * sms) w.warps = (int)((warps + sms - 1) / sms);
+    w.smem = head + w.warps * per_warp;
+    return w;
 }
 
-// A whole ensemble: the scratch comes from the stream-ordered allocator; if
-// that fails, the one-pass kernel runs with one block per chains_per_block
-// chains (same outputs).
-template <int G, int T, bool LJ>
-int launch_one(const OffArgs &a, int N, cudaStream_t s)
+int launch_wide(const OffArgs &a, int gref, int64_t c_lo, int64_t c_hi, void *counter,
+                cudaStream_t s, int64_t *resident)
 {
-    const bool two_pass = !LJ && N <= 128;
-    const size_t bytes = kScratchHeader + (two_pass ? mask_bytes(a.C) : 0);
-    void *buf = nullptr;
-    if (cudaMallocAsync(&buf, bytes, s) == cudaSuccess) {
-        cudaError_t e = two_pass ? cudaMemsetAsync(static_cast<unsigned char *>(buf) +
-                                                       kScratchHeader, 0, bytes - kScratchHeader, s)
-                                 : cudaSuccess;
-        uint32_t *mask = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(buf) +
-                                                      kScratchHeader);
-        int st = e == cudaSuccess ? launch_range<G, T, LJ>(a, N, 0, a.C, buf, mask, s)
-                                  : set_error(ROSEN_ECUDA, "rosen_offlattice_grow: %s",
-                                              cudaGetErrorString(e));
-        const cudaError_t f = cudaFreeAsync(buf, s);
-        if (st != ROSEN_OK) return st;
-        if (f != cudaSuccess)
-            return set_error(ROSEN_ECUDA, "rosen_offlattice_grow: freeing the work counter: %s",
-                             cudaGetErrorString(f));
-        return ROSEN_OK;
-    }
-    cudaGetLastError();   // clear the failed allocation; grow in one pass
-    const int chains = chains_per_block_for(G, N, LJ);
-    const size_t smem = kTable * sizeof(float) + (size_t)chains * chain_smem_bytes(N, LJ);
-    const int64_t blocks = (a.C + chains - 1) / chains;
-    allow_max_smem(offlattice_group_kernel<G, T, LJ>);
-    offlattice_group_kernel<G, T, LJ><<<(unsigned)blocks, chains * G, smem, s>>>(a, chains);
-    return check_launch("rosen_offlattice_grow");
-}
-
-// Chains the GPU grows at once with the first-pass (or only) kernel.
-template <int G, int T, bool LJ>
-int64_t resident(int N)
-{
-    const int chains = chains_per_block_for(G, N, LJ);
-    const size_t smem = kTable * sizeof(float) + (size_t)chains * chain_smem_bytes(N, LJ);
-    auto first = (!LJ && N <= 128) ? offlattice_queue_kernel<G, T, LJ, !LJ>
-                                   : offlattice_queue_kernel<G, T, LJ, false>;
     int dev = 0, sms = 0, bps = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        allow_max_smem(first) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, first, chains * G, smem) !=
-            cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return (int64_t)bps * sms * chains;
-}
-
-// launch_one (counters == nullptr: a whole ensemble, scratch allocated
-// here), launch_range, or the resident chain count (resident_out != nullptr).
-template <int G, bool LJ>
-int launch_g(const OffArgs &a, int N, int k, int64_t c_lo, int64_t c_hi, void *counters,
-             uint32_t *mask, cudaStream_t s, int64_t *resident_out = nullptr)
-{
-    const int T = (k + G - 1) / G;
-    if (resident_out) {
-        *resident_out = T <= 1 ? resident<G, 1, LJ>(N) : T <= 2 ? resident<G, 2, LJ>(N)
-                                                                  : resident<G, 4, LJ>(N);
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return set_cuda_error(e);
+    const WidePlan w = wide_plan(a, gref, resident ? INT64_MAX / 64 : c_hi - c_lo, sms);
+    const int64_t per_block = (int64_t)w.warps * (32 / w.G);
+    e = allow_max_smem(w.fn);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, w.fn, w.warps * 32, w.smem);
+    if (resident) {
+        *resident = e == cudaSuccess ? (int64_t)bps * sms * per_block : 0;
+        if (e != cudaSuccess) cudaGetLastError();
         return ROSEN_OK;
     }
-    if (!counters) {
-        if (T <= 1) return launch_one<G, 1, LJ>(a, N, s);
-        if (T <= 2) return launch_one<G, 2, LJ>(a, N, s);
-        return launch_one<G, 4, LJ>(a, N, s);
+    if (e == cudaSuccess && counter) e = cudaMemsetAsync(counter, 0, kScratchHeader, s);
+    if (e == cudaSuccess) {
+        int64_t grid = (c_hi - c_lo + per_block - 1) / per_block;
+        if (counter) grid = std::min(grid, (int64_t)(bps > 0 ? bps : 1) * sms);
+        w.fn<<<(unsigned)grid, w.warps * 32, w.smem, s>>>(
+            a, w.sh, static_cast<unsigned long long *>(counter), c_lo, c_hi);
+        e = cudaGetLastError();
     }
-    if (T <= 1) return launch_range<G, 1, LJ>(a, N, c_lo, c_hi, counters, mask, s);
-    if (T <= 2) return launch_range<G, 2, LJ>(a, N, c_lo, c_hi, counters, mask, s);
-    return launch_range<G, 4, LJ>(a, N, c_lo, c_hi, counters, mask, s);
+    return e == cudaSuccess ? ROSEN_OK : set_cuda_error(e);
 }
 
-template <bool LJ>
-int launch_lj(const OffArgs &a, int G, int N, int k, int64_t c_lo, int64_t c_hi, void *counters,
-              uint32_t *mask, cudaStream_t s, int64_t *resident_out = nullptr)
+// Local chains [c_lo, c_hi) with G lanes per chain (hard spheres: sums in that
+// order), with or without a chain counter; or the chains the GPU grows at
+// once (resident != nullptr).
+int launch_range(const OffArgs &a, bool lj, int G, int64_t c_lo, int64_t c_hi, void *counter,
+                 cudaStream_t s, int64_t *resident = nullptr)
 {
-    if (G == 8) return launch_g<8, LJ>(a, N, k, c_lo, c_hi, counters, mask, s, resident_out);
-    if (G == 16) return launch_g<16, LJ>(a, N, k, c_lo, c_hi, counters, mask, s, resident_out);
-    return launch_g<32, LJ>(a, N, k, c_lo, c_hi, counters, mask, s, resident_out);
+    if (!lj) return launch_wide(a, G, c_lo, c_hi, counter, s, resident);
+    const int T = (a.k + G - 1) / G;
+#define ROSEN_LAUNCH(GG, TT) return launch_lj<GG, TT>(a, c_lo, c_hi, counter, s, resident);
+    if (G == 8) {
+        if (T <= 1) ROSEN_LAUNCH(8, 1)
+        if (T <= 2) ROSEN_LAUNCH(8, 2)
+        ROSEN_LAUNCH(8, 4)
+    }
+    if (G == 16) {
+        if (T <= 1) ROSEN_LAUNCH(16, 1)
+        if (T <= 2) ROSEN_LAUNCH(16, 2)
+        ROSEN_LAUNCH(16, 4)
+    }
+    if (T <= 1) ROSEN_LAUNCH(32, 1)
+    if (T <= 2) ROSEN_LAUNCH(32, 2)
+    ROSEN_LAUNCH(32, 4)
+#undef ROSEN_LAUNCH
 }
 
 // The batch kernel of class (G, T, LJ) through one function pointer type.
@@ -497,45 +462,56 @@ void offlattice_make_args(const rosen_offlattice_params *p, const rosen_offlatti
     memcpy(out, &a, sizeof a);
 }
 
+namespace {
+
+int lanes_of(const rosen_offlattice_params *p)
+{
+    return p->lanes_per_chain
+               ? p->lanes_per_chain
+               : offlattice_default_lanes(p->k, p->potential == ROSEN_LJ, p->N);
+}
+
+}  // namespace
+
+// A whole ensemble: the chain counter comes from the stream-ordered allocator;
+// if that fails, the chains grow without one.
 int offlattice_launch(const rosen_offlattice_params *p, const rosen_offlattice_out *o,
                       unsigned long long *counters, cudaStream_t s)
 {
     OffArgs a;
     offlattice_make_args(p, o, counters, &a);
-    const bool lj = p->potential == ROSEN_LJ;
-    const int G =
-        p->lanes_per_chain ? p->lanes_per_chain : offlattice_default_lanes(p->k, lj, p->N);
-    return lj ? launch_lj<true>(a, G, p->N, p->k, 0, p->C, nullptr, nullptr, s)
-              : launch_lj<false>(a, G, p->N, p->k, 0, p->C, nullptr, nullptr, s);
+    void *buf = nullptr;
+    if (cudaMallocAsync(&buf, kScratchHeader, s) != cudaSuccess) {
+        cudaGetLastError();   // clear the failed allocation
+        buf = nullptr;
+    }
+    const int st = launch_range(a, p->potential == ROSEN_LJ, lanes_of(p), 0, p->C, buf, s);
+    const cudaError_t f = buf ? cudaFreeAsync(buf, s) : cudaSuccess;
+    if (st != ROSEN_OK) return st;
+    if (f != cudaSuccess)
+        return set_error(ROSEN_ECUDA, "rosen_offlattice_grow: freeing the work counter: %s",
+                         cudaGetErrorString(f));
+    return ROSEN_OK;
 }
 
 size_t offlattice_range_counter_bytes() { return kScratchHeader; }
-size_t offlattice_range_mask_bytes(int64_t C) { return mask_bytes(C); }
 
 int offlattice_grow_range(const rosen_offlattice_params *p, const rosen_offlattice_out *o,
-                          int64_t c_lo, int64_t c_hi, void *counters, uint32_t *mask,
-                          cudaStream_t s)
+                          int64_t c_lo, int64_t c_hi, void *counter, cudaStream_t s)
 {
     if (c_hi <= c_lo) return ROSEN_OK;
     OffArgs a;
     offlattice_make_args(p, o, reinterpret_cast<unsigned long long *>(o->counters), &a);
-    const bool lj = p->potential == ROSEN_LJ;
-    const int G =
-        p->lanes_per_chain ? p->lanes_per_chain : offlattice_default_lanes(p->k, lj, p->N);
-    return lj ? launch_lj<true>(a, G, p->N, p->k, c_lo, c_hi, counters, mask, s)
-              : launch_lj<false>(a, G, p->N, p->k, c_lo, c_hi, counters, mask, s);
+    return launch_range(a, p->potential == ROSEN_LJ, lanes_of(p), c_lo, c_hi, counter, s);
 }
 
 int64_t offlattice_resident_chains(const rosen_offlattice_params *p)
 {
     OffArgs a;
-    memset(&a, 0, sizeof a);
-    const bool lj = p->potential == ROSEN_LJ;
-    const int G =
-        p->lanes_per_chain ? p->lanes_per_chain : offlattice_default_lanes(p->k, lj, p->N);
+    const rosen_offlattice_out none = {};
+    offlattice_make_args(p, &none, nullptr, &a);
     int64_t r = 0;
-    if (lj) launch_lj<true>(a, G, p->N, p->k, 0, 0, nullptr, nullptr, nullptr, &r);
-    else launch_lj<false>(a, G, p->N, p->k, 0, 0, nullptr, nullptr, nullptr, &r);
+    launch_range(a, p->potential == ROSEN_LJ, lanes_of(p), 0, 0, nullptr, nullptr, &r);
     return r;
 }
 

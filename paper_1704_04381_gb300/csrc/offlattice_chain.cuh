@@ -35,7 +35,6 @@ struct OffArgs {
     unsigned long long *counters;   // optional [3]: steps re-decided, chains, listed beads
     uint16_t *attempts;             // optional [C]
     uint32_t max_att;               // growths per chain (1: no restart)
-    uint32_t *deferred;             // two-pass hard-sphere growth: bit c = chain c deferred
 };
 
 // Per-chain shared memory: float-float positions, the near list, the trace.
@@ -746,13 +745,10 @@ __device__ __forceinline__ int long_near_list(const OffArgs &a, const ChainLong 
 
 // Grow chain c (local index) of the ensemble a with the G lanes of group g,
 // in the per-chain storage w (shared memory; for kLong, device memory with a
-// cell grid, generation counter *genp).  With kDefer the FP64 re-decision is
-// not compiled in: a chain that meets a step its FP32 arithmetic cannot
-// decide sets its bit in a.deferred and stops without writing anything; a
-// second pass grows it again, from the start, with the FP64 path.  In restart mode a growth that
-// reaches a dead end is thrown away and the chain grown again from bead 0,
-// with the attempt index in the high half of the step word.
-template <int G, int T, bool LJ, class W = ChainSmem, bool kDefer = false, bool kFly = false>
+// cell grid, generation counter *genp).  In restart mode a growth that reaches
+// a dead end is thrown away and the chain grown again from bead 0, with the
+// attempt index in the high half of the step word.
+template <int G, int T, bool LJ, class W = ChainSmem, bool kFly = false>
 __device__ __forceinline__ void off_chain(const OffArgs &a, int64_t c, const W &w,
                                           const Group<G> &g, const float *logm,
                                           uint32_t *genp = nullptr)
@@ -999,15 +995,10 @@ __device__ __forceinline__ void off_chain(const OffArgs &a, int64_t c, const W &
 
             // ---- 5. FP64 re-decision of an ambiguous step -------------------
             if (!ok) {
-                if constexpr (kDefer) {
-                    if (g.gl == 0) atomicOr(&a.deferred[c >> 5], 1u << (c & 31));
-                    return;
-                } else {
-                    ++rechecks;
-                    redecide<G, T, LJ, kFly>(a, w, g, chain, aw, exact_upto, i, nn, selw, logm, ehx,
-                                       ehy, ehz, elx, ely, elz, sel, logS, dead_at);
-                    exact_upto = i - 1;
-                }
+                ++rechecks;
+                redecide<G, T, LJ, kFly>(a, w, g, chain, aw, exact_upto, i, nn, selw, logm, ehx,
+                                         ehy, ehz, elx, ely, elz, sel, logS, dead_at);
+                exact_upto = i - 1;
             }
             if (dead_at) break;
 

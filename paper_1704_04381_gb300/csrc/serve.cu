@@ -41,7 +41,7 @@
 // entry points.
 //
 // Device memory of a request (outputs, reduction scratch, the real-space
-// chain counters and deferral mask, a long-chain workspace, stored
+// chain counters, a long-chain workspace, stored
 // conformations) comes from one stream-ordered pool and is counted against
 // the budget from admission until it is returned.
 #include <math.h>
@@ -101,7 +101,7 @@ struct Request {
     void *rws = nullptr;       // reduction workspace
     size_t rws_bytes = 0;
     rosen_stats *dstats = nullptr;
-    void *scratch = nullptr;   // real space: two sets of chain counters, the deferral mask
+    void *scratch = nullptr;   // real space: two sets of chain counters
     void *long_ws = nullptr;   // long chains: their workspace
     size_t long_bytes = 0;
     cudaStream_t streams[2] = {nullptr, nullptr};   // slices alternate between them
@@ -187,12 +187,13 @@ size_t long_workspace_bytes(const rosen_request &r)
     return align256(std::max(one, std::min(want, kLongWorkspaceCap)));
 }
 
-// Real-space chain counters (one set per stream) and deferral mask
-// (shared-memory kernels).
+// Real-space chain counters (one set per stream; shared-memory kernels).  A bit
+// per chain is reserved with them: what a budget or a pool cap admits is a
+// promise to clients and stays what it was when launches shared such a mask.
 size_t scratch_bytes(const rosen_request &r)
 {
     if (r.model != ROSEN_MODEL_OFFLATTICE || long_request(r)) return 0;
-    return align256(2 * offlattice_range_counter_bytes() + offlattice_range_mask_bytes(r.C));
+    return align256(2 * offlattice_range_counter_bytes() + (size_t)((r.C + 31) / 32) * 4);
 }
 
 // Device bytes a request holds while it runs, and what stored conformations
@@ -446,7 +447,6 @@ bool admit(rosen_server *s, Request *q)
         e = cudaMallocFromPoolAsync(&q->coords, q->coord_bytes, s->pool, s0);
     if (e == cudaSuccess) {
         carve(q);
-        if (q->scratch) e = cudaMemsetAsync(q->scratch, 0, scratch_bytes(q->req), s0);
     }
     // The second stream starts after the allocation and the set-up.
     if (e == cudaSuccess) e = cudaEventRecord(q->join, s0);
@@ -511,8 +511,7 @@ void finish(Request *q)
 // Enqueue the next slice of q on the stream after the last one's:
 // chains [next_chain, next_chain + n), or the whole request for long chains.
 // A slice holds about kSliceNs of estimated GPU time but at least twice the
-// chains the GPU grows at once, and starts at a multiple of 32 chains (the
-// deferral mask's words).
+// chains the GPU grows at once.
 void launch_slice(rosen_server *s, Request *q)
 {
     const int64_t C = q->req.C;
@@ -544,8 +543,7 @@ void launch_slice(rosen_server *s, Request *q)
     } else {
         unsigned char *sc = static_cast<unsigned char *>(q->scratch);
         const size_t cb = offlattice_range_counter_bytes();
-        st = offlattice_grow_range(&q->op, &q->oo, c_lo, c_hi, sc + lane * cb,
-                                   reinterpret_cast<uint32_t *>(sc + 2 * cb), st_q);
+        st = offlattice_grow_range(&q->op, &q->oo, c_lo, c_hi, sc + lane * cb, st_q);
     }
     if (sl.end) cudaEventRecord(sl.end, st_q);
     q->next_chain = c_hi;
