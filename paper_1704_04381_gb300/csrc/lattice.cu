@@ -34,6 +34,7 @@
 
 #include "common.cuh"
 #include "internal.cuh"
+#include "lattice_blocks.cuh"
 #include "lattice_step.cuh"
 
 namespace rosen {
@@ -723,6 +724,48 @@ int lattice_retry_launch(const LatticeArgs &a, int N, int B, int64_t c_lo, int64
     return check_launch("rosen_lattice_grow");
 }
 
+// Chains from this length on grow with bitmap tables (lattice_blocks.cuh),
+// which overtake the scan between N = 128 and 160, athermal and interacting.
+constexpr int kBlocksFromN = 160;
+
+// Their kernel's shape: blocks of one warp, and the warps the GPU holds at once.
+struct BlocksPlan {
+    void (*kern)(const LatticeArgs, int, int64_t, int64_t, int64_t);
+    int entries;
+    size_t smem;
+    int64_t resident;     // 0: a CUDA error
+};
+
+BlocksPlan blocks_plan(int N, bool isaw)
+{
+    BlocksPlan b;
+    b.kern = isaw ? lattice_blocks_kernel<true> : lattice_blocks_kernel<false>;
+    b.entries = site_entries(N);
+    b.smem = (size_t)b.entries * 12 * 32;
+    int bps = 0, dev = 0, sms = 0;
+    cudaError_t e = allow_max_smem(b.kern);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, b.kern, 32, b.smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    b.resident = e == cudaSuccess ? (int64_t)bps * sms : 0;
+    return b;
+}
+
+// Every warp takes an equal, contiguous share of the chains (at least one per
+// lane), so that all are resident at once.
+int lattice_blocks_launch(const LatticeArgs &a, int64_t c_lo, int64_t c_hi, cudaStream_t s)
+{
+    const BlocksPlan b = blocks_plan(a.N, a.isaw);
+    if (b.resident < 1)
+        return set_error(ROSEN_ECUDA, "rosen_lattice_grow: %s", cudaGetErrorString(cudaGetLastError()));
+    const int64_t n = c_hi - c_lo;
+    const int64_t per_warp = std::max<int64_t>(32, (n + b.resident - 1) / b.resident);
+    b.kern<<<(unsigned)((n + per_warp - 1) / per_warp), 32, b.smem, s>>>(a, b.entries, per_warp,
+                                                                         c_lo, c_hi);
+    return check_launch("rosen_lattice_grow");
+}
+
 // Grow local chains [c_lo, c_hi) of a validated ensemble (shared-memory
 // kernels, N <= 512).  Every chain's outputs are those of a call over all C
 // chains, bit for bit: a chain is grown by one lane whatever its block.
@@ -732,6 +775,7 @@ int lattice_grow_range(const rosen_lattice_params *p, const rosen_lattice_out *o
     if (c_hi <= c_lo) return ROSEN_OK;
     LatticeArgs a;
     lattice_make_args(p, o, &a);
+    if (p->N >= kBlocksFromN) return lattice_blocks_launch(a, c_lo, c_hi, s);
     const int B = lattice_block(p->N);
     if (a.max_att > 1) return lattice_retry_launch(a, p->N, B, c_lo, c_hi, s);
     const size_t smem = lattice_smem_bytes(p->N, B);
@@ -747,6 +791,11 @@ int lattice_grow_range(const rosen_lattice_params *p, const rosen_lattice_out *o
 
 int64_t lattice_resident_chains(const rosen_lattice_params *p)
 {
+    if (p->N >= kBlocksFromN) {
+        const int64_t warps = blocks_plan(p->N, p->beta_eps != 0.0).resident;
+        if (warps < 1) cudaGetLastError();
+        return 32 * warps;
+    }
     const int B = lattice_block(p->N);
     const size_t smem = lattice_smem_bytes(p->N, B);
     auto kern = p->beta_eps != 0.0
