@@ -2,15 +2,27 @@
 // (Guo & Baulin, Eq. 2 with W as the importance weight; Eq. 9 for Z_N).
 //
 // Rosenbluth weights span hundreds of orders of magnitude, so the sums are
-// formed in FP64 relative to a running maximum (log-sum-exp).  The chains
-// are cut into fixed tiles of kTile chains; one block reduces one tile to a
-// partial (its max M_t and the sums scaled by exp(-M_t)), and a single block
-// merges the partials.  Tiles, the in-tile order and the merge tree depend
-// only on C, so the result is bit-for-bit deterministic.
+// formed in FP64 relative to a maximum (log-sum-exp).  The chains are cut into
+// fixed tiles of kTile chains; a cluster of kTileCtas blocks reduces one tile
+// to a partial (its max M_t and the sums scaled by exp(-M_t)), and a cluster
+// of kFinalCtas blocks merges an ensemble's partials: their maximum first, then
+// every partial scaled once.  Tiles, the in-tile order and the merge order
+// depend only on C, so the result is bit-for-bit deterministic.
+//
+// Bound by the FP64 pipe (a warp instruction takes it 16 cycles) for many
+// chains and by latency for few.  So a tile is spread over four SMs, the block
+// sums go through shared memory (a hundred warp instructions where shuffles
+// took 360), the weights' exponential takes 10 FP64 operations, and the merge
+// takes one exponential per partial instead of two per pair merged and forms
+// the statistics on different lanes.  GB300, one block per tile and a tree of
+// pairwise merges before, and now: 10^5 chains 59.5 -> 26.7 us, 10^7 chains
+// 0.957 -> 0.710 ms (weights from counts 1.130 -> 0.807 ms).
 #include <math.h>
 #include <string.h>
 
 #include <mutex>
+
+#include <cooperative_groups.h>
 
 #include "common.cuh"
 #include "internal.cuh"
@@ -18,10 +30,14 @@
 namespace rosen {
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kTile = 2048;
-constexpr int kThreads = 256;
-constexpr int kPerThread = kTile / kThreads;
-constexpr int kFinalThreads = 256;
+constexpr int kTileCtas = 4;
+constexpr int kThreads = 128;
+constexpr int kPerThread = kTile / kTileCtas / kThreads;
+constexpr int kFinalCtas = 8;
+constexpr int kSums = 10;      // the eight sums, live chains, growths
 
 struct Partial {
     double M;          // max log W in the tile (-inf: no live chain)
@@ -54,12 +70,12 @@ __device__ __forceinline__ void load_chain(const ReduceArgs &a, int64_t c, doubl
             if (v.x & 0xFFFFu) {
                 lw = -INFINITY;
             } else {
-                // log W = sum_m counts[m] log m, exact up to FP64 rounding.
-                const uint32_t cm[7] = {v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16,
-                                        v.z & 0xFFFFu, v.z >> 16, v.w & 0xFFFFu};
-                double s = 0.0;
-#pragma unroll
-                for (int q = 2; q <= 6; ++q) s = fma((double)cm[q], a.logm[q], s);
+                // log W = sum_m counts[m] log m over the primes of m = 2 .. 6,
+                // exact up to FP64 rounding.
+                const uint32_t c2 = v.y & 0xFFFFu, c3 = v.y >> 16, c4 = v.z & 0xFFFFu,
+                               c5 = v.z >> 16, c6 = v.w & 0xFFFFu;
+                const double s = fma((double)(c2 + 2u * c4 + c6), a.logm[2],
+                                     fma((double)(c3 + c6), a.logm[3], (double)c5 * a.logm[5]));
                 lw = s;
             }
         } else {
@@ -74,9 +90,52 @@ __device__ __forceinline__ void load_chain(const ReduceArgs &a, int64_t c, doubl
     }
 }
 
-// Merge partial b into a (same max-shift convention).  Host and device: the
-// multi-GPU merge (rosen_stats_merge) uses the same arithmetic.
-__host__ __device__ __forceinline__ void merge(double &Ma, double *sa, double &na, double Mb,
+// exp(x) for the weights, x <= 0: the table-driven method of Tang (ACM Trans.
+// Math. Softw. 15 (1989) 144).  x = (64 k + j) ln2 / 64 + r with |r| <= ln2 / 128;
+// exp(x) = 2^k 2^(j/64) (1 + p(r)), p the Taylor polynomial of e^r - 1 to r^5
+// (remainder below 4e-17), 2^(j/64) from a table; 10 FP64 operations.  Below
+// -700, and for NaN, the library's exp.
+constexpr double kInvStep = 0x1.71547652b82fep+6;        // 64 / ln 2
+constexpr double kStepHi = 0x1.62e42fefa0000p-7;         // ln 2 / 64: 38 bits, and the rest
+constexpr double kStepLo = 0x1.cf79abc9e3b3ap-46;
+__constant__ const double kPow2[64] = {   // 2^(j / 64)
+    0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
+    0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
+    0x1.172b83c7d517bp+0, 0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
+    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0, 0x1.2d285a6e4030bp+0,
+    0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0, 0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0,
+    0x1.3dea64c123422p+0, 0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
+    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0, 0x1.56f4736b527dap+0,
+    0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0, 0x1.6247eb03a5585p+0, 0x1.6623882552225p+0,
+    0x1.6a09e667f3bcdp+0, 0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
+    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0, 0x1.868d99b4492edp+0,
+    0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0, 0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0,
+    0x1.9c49182a3f090p+0, 0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
+    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0, 0x1.bcc1e904bc1d2p+0,
+    0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0, 0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0,
+    0x1.d5818dcfba487p+0, 0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
+    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0, 0x1.fa7c1819e90d8p+0,
+};
+
+// (At most one ulp from the library's exp on 3 10^7 arguments in [-700, 0].)
+__device__ __forceinline__ double exp_weight(double x, const double *pow2)
+{
+    if (!(x > -700.0)) return exp(x);
+    constexpr double kRound = 0x1.8p52;
+    const double t = fma(x, kInvStep, kRound);
+    const int n = __double2loint(t);
+    const double f = t - kRound;
+    const double r = fma(f, -kStepLo, fma(f, -kStepHi, x));
+    const double p = fma(r * r, fma(r, fma(r, fma(r, 1.0 / 120.0, 1.0 / 24.0), 1.0 / 6.0), 0.5), r);
+    const double y = pow2[n & 63];
+    const double e = fma(y, p, y);
+    // (k >= -1011: the scaled exponent field stays positive.)
+    return __hiloint2double(__double2hiint(e) + ((n >> 6) << 20), __double2loint(e));
+}
+
+// Merge the sums of chain set b into those of a (same max-shift convention):
+// the multi-GPU merge (rosen_stats_merge).
+inline void merge(double &Ma, double *sa, double &na, double Mb,
                                                const double *sb, double nb)
 {
     const double M = fmax(Ma, Mb);
@@ -94,11 +153,12 @@ __host__ __device__ __forceinline__ void merge(double &Ma, double *sa, double &n
     na += nb;
 }
 
-// The statistics of an ensemble from its merged sums: Eq. 9's log Z (mean
+// The statistics of an ensemble from its merged sums (on the host; finish_warp
+// is the device's form): Eq. 9's log Z (mean
 // weight over the n growths), Eq. 2's W-weighted means of R_ee^2 and R_g^2,
 // their ratio standard errors sqrt(sum w^2 (A - mean)^2) / sum w, and the
 // effective sample size (sum w)^2 / sum w^2.
-__host__ __device__ __forceinline__ rosen_stats finish(double M, const double *S, double alive,
+inline rosen_stats finish(double M, const double *S, double alive,
                                                        double n, int N, int k)
 {
     rosen_stats r;
@@ -133,147 +193,243 @@ __host__ __device__ __forceinline__ rosen_stats finish(double M, const double *S
     return r;
 }
 
-// Reduce tile `tile` of the ensemble a into *out (one block of kThreads).
+// Sums of the block's kSums values per thread, in a fixed order: thread q of
+// sum q / kSegs adds a segment of the threads' values one after another, and
+// the segments are added in pairs.  The result is in v[0..kSums) of shared
+// memory when the call returns.
+constexpr int kSegs = 8;
+struct BlockSums {
+    double part[kSums][kThreads + kSegs];   // (a word of padding per segment)
+    double v[kSums];
+};
+
+__device__ __forceinline__ void block_sums(BlockSums &b, const double (&s)[kSums])
+{
+    constexpr int kSeg = kThreads / kSegs;
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int q = 0; q < kSums; ++q) b.part[q][t + t / kSeg] = s[q];
+    __syncthreads();
+    if (t < kSums * kSegs) {
+        const double *x = &b.part[t / kSegs][(t % kSegs) * (kSeg + 1)];
+        double y = x[0];
+#pragma unroll
+        for (int q = 1; q < kSeg; ++q) y += x[q];
+        b.part[t / kSegs][(t % kSegs) * (kSeg + 1)] = y;
+    }
+    __syncthreads();
+    if (t < kSums) {
+        const double *x = b.part[t];
+        double y[kSegs];
+#pragma unroll
+        for (int q = 0; q < kSegs; ++q) y[q] = x[q * (kSeg + 1)];
+#pragma unroll
+        for (int o = kSegs / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < o; ++q) y[q] += y[q + o];
+        b.v[t] = y[0];
+    }
+    __syncthreads();
+}
+
+// Maximum over the block, in every thread.
+__device__ __forceinline__ double block_max(double m, double *warp_max)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
+    __syncthreads();
+    m = warp_max[0];
+#pragma unroll
+    for (int w = 1; w < kThreads / 32; ++w) m = fmax(m, warp_max[w]);
+    return m;
+}
+
+// Reduce tile `tile` of the ensemble a into *out (one cluster; block r of it
+// takes the tile's r-th quarter).
 __device__ __forceinline__ void reduce_tile(const ReduceArgs &a, int64_t tile, Partial *out)
 {
-    __shared__ double red[kThreads / 32][10];   // 9 sums + the growth count
-    __shared__ double tileM;
-    const int64_t c0 = tile * kTile;
+    __shared__ BlockSums b;
+    __shared__ double warp_max[kThreads / 32], block_m, pow2[64];
+    if (threadIdx.x < 64) pow2[threadIdx.x] = kPow2[threadIdx.x];
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int64_t c0 = tile * kTile + (int64_t)rank * (kTile / kTileCtas);
     double lw[kPerThread], A1[kPerThread], A2[kPerThread];
     double m = -INFINITY;
-    double growths = 0.0;   // Eq. 9's sample size: chains, or attempts in restart mode
+    uint32_t growths = 0u;   // Eq. 9's sample size: chains, or attempts in restart mode
 #pragma unroll
     for (int q = 0; q < kPerThread; ++q) {
         const int64_t c = c0 + threadIdx.x + (int64_t)q * kThreads;
         if (c < a.C) {
             load_chain(a, c, lw[q], A1[q], A2[q]);
-            growths += a.attempts ? (double)a.attempts[c] : 1.0;
+            growths += a.attempts ? a.attempts[c] : 1u;
         } else {
             lw[q] = -INFINITY;
             A1[q] = A2[q] = 0.0;
         }
         m = fmax(m, lw[q]);
     }
-    // Block maximum.
+    m = block_max(m, warp_max);
+    if (threadIdx.x == 0) block_m = m;
+    cluster.sync();
+    double M = *cluster.map_shared_rank(&block_m, 0);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, off));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) red[warp][0] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double mm = -INFINITY;
-        for (int w = 0; w < kThreads / 32; ++w) mm = fmax(mm, red[w][0]);
-        tileM = mm;
-    }
-    __syncthreads();
-    const double M = tileM;
-    double s[9];
+    for (int r = 1; r < kTileCtas; ++r) M = fmax(M, *cluster.map_shared_rank(&block_m, r));
+    double s[kSums];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) s[q] = 0.0;
+    for (int q = 0; q < kSums; ++q) s[q] = 0.0;
+    uint32_t alive = 0u;
     if (M > -INFINITY) {
 #pragma unroll
         for (int q = 0; q < kPerThread; ++q) {
             if (lw[q] == -INFINITY) continue;
-            const double w = exp(lw[q] - M), w2 = w * w;
+            const double w = exp_weight(lw[q] - M, pow2), w2 = w * w;
+            const double u = w2 * A1[q], v = w2 * A2[q];
             s[0] += w;
             s[1] += w * A1[q];
             s[2] += w * A2[q];
             s[3] += w2;
-            s[4] += w2 * A1[q];
-            s[5] += w2 * A1[q] * A1[q];
-            s[6] += w2 * A2[q];
-            s[7] += w2 * A2[q] * A2[q];
-            s[8] += 1.0;
+            s[4] += u;
+            s[5] += u * A1[q];
+            s[6] += v;
+            s[7] += v * A2[q];
+            ++alive;
         }
     }
+    s[8] = (double)alive;
+    s[9] = (double)growths;
+    block_sums(b, s);
+    cluster.sync();
+    if (rank == 0 && threadIdx.x < kSums) {
+        double t = b.v[threadIdx.x];
 #pragma unroll
-    for (int q = 0; q < 9; ++q)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], off);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) growths += __shfl_xor_sync(0xffffffffu, growths, off);
-    __syncthreads();
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < 9; ++q) red[warp][q] = s[q];
-        red[warp][9] = growths;
+        for (int r = 1; r < kTileCtas; ++r) t += *cluster.map_shared_rank(&b.v[threadIdx.x], r);
+        double *field = threadIdx.x < 8 ? &out->s[threadIdx.x]
+                                        : (threadIdx.x == 8 ? &out->alive : &out->n);
+        *field = t;
+        if (threadIdx.x == 0) out->M = M;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        Partial P;
-        P.M = M;
-        for (int q = 0; q < 8; ++q) {
-            double t = 0.0;
-            for (int w = 0; w < kThreads / 32; ++w) t += red[w][q];
-            P.s[q] = t;
-        }
-        double al = 0.0, ng = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) {
-            al += red[w][8];
-            ng += red[w][9];
-        }
-        P.alive = al;
-        P.n = ng;
-        P.pad = 0.0;
-        *out = P;
-    }
+    cluster.sync();      // (no block leaves while its sums are read)
 }
 
-__global__ void __launch_bounds__(kThreads) reduce_tiles_kernel(const ReduceArgs a, Partial *part)
+__global__ void __cluster_dims__(kTileCtas) __launch_bounds__(kThreads)
+    reduce_tiles_kernel(const ReduceArgs a, Partial *part)
 {
-    reduce_tile(a, blockIdx.x, &part[blockIdx.x]);
+    const int64_t t = blockIdx.x / kTileCtas;
+    reduce_tile(a, t, &part[t]);
 }
 
-// Merge the ntiles partials of one ensemble in a fixed tree (one block).
+// finish() by one warp: the divisions, logarithms and square roots of
+// different statistics on different lanes, so that a chain of four of them is
+// waited for and not of ten.  S: S0 .. Q2b, live chains, growths.
+__device__ __forceinline__ void finish_warp(double M, const double *S, int N, int k, rosen_stats *out)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const double alive = S[8], n = S[9];
+    if (alive == 0.0) {
+        if (lane == 0) {
+            rosen_stats r;
+            r.n = n;
+            r.n_alive = alive;
+            r.log_max = M;
+            r.S0 = r.S1 = r.S2 = r.Q0 = r.Q1_r2 = r.Q2_r2 = r.Q1_rg2 = r.Q2_rg2 = 0.0;
+            r.logZ = r.logZ_norm = -INFINITY;
+            r.mean_r2 = r.se_r2 = r.mean_rg2 = r.se_rg2 = NAN;
+            r.ess = 0.0;
+            *out = r;
+        }
+        return;
+    }
+    // Lanes 0, 1: mean and standard error of R_ee^2, R_g^2; 2: log Z; 3: ESS.
+    const int a = lane & 1;
+    const double num = lane == 3 ? S[0] * S[0] : (lane == 2 ? S[0] : S[1 + a]);
+    const double den = lane == 3 ? S[3] : (lane == 2 ? n : S[0]);
+    const double q = num / den;
+    const double v = S[5 + 2 * a] - 2.0 * q * S[4 + 2 * a] + q * q * S[3];
+    const double se = sqrt(v > 0.0 ? v : 0.0) / S[0];
+    const double lg = log(lane == 3 ? (double)max(k, 1) : q);
+    const double logk = __shfl_sync(kAll, lg, 3);
+    if (lane < 2) {
+        (lane ? out->mean_rg2 : out->mean_r2) = q;
+        (lane ? out->se_rg2 : out->se_r2) = se;
+    } else if (lane == 2) {
+        const double z = M + lg;
+        out->logZ = z;
+        out->logZ_norm = k > 0 ? z - (double)(N - 1) * logk : z;
+    } else if (lane == 3) {
+        out->ess = q;
+        out->n = n;
+        out->n_alive = alive;
+        out->log_max = M;
+    } else if (lane < 12) {
+        (&out->S0)[lane - 4] = S[lane - 4];      // S0 .. Q2_rg2 follow one another
+    }
+}
+
+// Merge the ntiles partials of one ensemble (one cluster): their maximum M,
+// then the sum of every partial's sums scaled by exp(M_t - M) (squared for the
+// sums of w^2).
 __device__ __forceinline__ void reduce_final(const Partial *part, int64_t ntiles,
                                              const ReduceArgs &a, rosen_stats *out)
 {
-    __shared__ double sM[kFinalThreads], sS[kFinalThreads][8], sN[kFinalThreads];
-    __shared__ double sG[kFinalThreads];
-    double M = -INFINITY, S[8] = {0, 0, 0, 0, 0, 0, 0, 0}, na = 0.0, ng = 0.0;
-    for (int64_t t = threadIdx.x; t < ntiles; t += kFinalThreads) {
-        merge(M, S, na, part[t].M, part[t].s, part[t].alive);
-        ng += part[t].n;
+    __shared__ BlockSums b;
+    __shared__ double warp_max[kThreads / 32], block_m;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int64_t t0 = (int64_t)rank * kThreads + threadIdx.x;
+    constexpr int64_t kStep = (int64_t)kFinalCtas * kThreads;
+    double M = -INFINITY;
+    for (int64_t t = t0; t < ntiles; t += kStep) M = fmax(M, part[t].M);
+    M = block_max(M, warp_max);
+    if (threadIdx.x == 0) block_m = M;
+    cluster.sync();
+#pragma unroll
+    for (int r = 0; r < kFinalCtas; ++r) M = fmax(M, *cluster.map_shared_rank(&block_m, r));
+    double s[kSums];
+#pragma unroll
+    for (int q = 0; q < kSums; ++q) s[q] = 0.0;
+    for (int64_t t = t0; t < ntiles; t += kStep) {
+        const Partial &p = part[t];
+        if (p.M > -INFINITY) {
+            const double f = exp(p.M - M), f2 = f * f;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) s[q] += p.s[q] * f;
+#pragma unroll
+            for (int q = 3; q < 8; ++q) s[q] += p.s[q] * f2;
+        }
+        s[8] += p.alive;
+        s[9] += p.n;
     }
-    sM[threadIdx.x] = M;
-    for (int q = 0; q < 8; ++q) sS[threadIdx.x][q] = S[q];
-    sN[threadIdx.x] = na;
-    sG[threadIdx.x] = ng;
-    __syncthreads();
-    for (int half = kFinalThreads / 2; half > 0; half >>= 1) {
-        if (threadIdx.x < half) {
-            double Mb = sM[threadIdx.x + half], Sb[8];
-            for (int q = 0; q < 8; ++q) Sb[q] = sS[threadIdx.x + half][q];
-            double Ma = sM[threadIdx.x], Sa[8], nA = sN[threadIdx.x];
-            for (int q = 0; q < 8; ++q) Sa[q] = sS[threadIdx.x][q];
-            merge(Ma, Sa, nA, Mb, Sb, sN[threadIdx.x + half]);
-            sM[threadIdx.x] = Ma;
-            for (int q = 0; q < 8; ++q) sS[threadIdx.x][q] = Sa[q];
-            sN[threadIdx.x] = nA;
-            sG[threadIdx.x] += sG[threadIdx.x + half];
+    block_sums(b, s);
+    cluster.sync();
+    if (rank == 0) {
+        if (threadIdx.x < kSums) {
+            double t = b.v[threadIdx.x];
+            for (int r = 1; r < kFinalCtas; ++r) t += *cluster.map_shared_rank(&b.v[threadIdx.x], r);
+            b.part[0][threadIdx.x] = t;
         }
         __syncthreads();
+        // The growth count is a sum of integer-valued partials: exact in FP64.
+        if (threadIdx.x < 32) finish_warp(M, b.part[0], a.N, a.k, out);
     }
-    if (threadIdx.x != 0) return;
-    // The growth count is a sum of integer-valued partials: exact in FP64.
-    *out = finish(sM[0], sS[0], sN[0], sG[0], a.N, a.k);
+    cluster.sync();      // (no block leaves while its sums are read)
 }
 
-__global__ void __launch_bounds__(kFinalThreads) reduce_final_kernel(const Partial *part,
-                                                                     int64_t ntiles,
-                                                                     const ReduceArgs a,
-                                                                     rosen_stats *out)
+__global__ void __cluster_dims__(kFinalCtas) __launch_bounds__(kThreads)
+    reduce_final_kernel(const Partial *part, int64_t ntiles, const ReduceArgs a, rosen_stats *out)
 {
     reduce_final(part, ntiles, a, out);
 }
 
-// Batched: block b reduces global tile b; tile_off[e] .. tile_off[e+1]-1 are
+// Batched: cluster b reduces global tile b; tile_off[e] .. tile_off[e+1]-1 are
 // the tiles of ensemble e.
-__global__ void __launch_bounds__(kThreads) reduce_tiles_batch_kernel(const ReduceArgs *args,
-                                                                      const int64_t *tile_off,
-                                                                      int n_ens, Partial *part)
+__global__ void __cluster_dims__(kTileCtas) __launch_bounds__(kThreads)
+    reduce_tiles_batch_kernel(const ReduceArgs *args, const int64_t *tile_off, int n_ens,
+                              Partial *part)
 {
-    const int64_t b = blockIdx.x;
+    const int64_t b = blockIdx.x / kTileCtas;
     int lo = 0, hi = n_ens;            // largest e with tile_off[e] <= b
     while (hi - lo > 1) {
         const int mid = (lo + hi) / 2;
@@ -283,12 +439,11 @@ __global__ void __launch_bounds__(kThreads) reduce_tiles_batch_kernel(const Redu
     reduce_tile(args[lo], b - tile_off[lo], &part[b]);
 }
 
-__global__ void __launch_bounds__(kFinalThreads) reduce_final_batch_kernel(const Partial *part,
-                                                                           const int64_t *tile_off,
-                                                                           const ReduceArgs *args,
-                                                                           rosen_stats *out)
+__global__ void __cluster_dims__(kFinalCtas) __launch_bounds__(kThreads)
+    reduce_final_batch_kernel(const Partial *part, const int64_t *tile_off, const ReduceArgs *args,
+                              rosen_stats *out)
 {
-    const int e = blockIdx.x;
+    const int e = blockIdx.x / kFinalCtas;
     reduce_final(part + tile_off[e], tile_off[e + 1] - tile_off[e], args[e], out + e);
 }
 
@@ -326,8 +481,9 @@ void reduce_batch_launch(const void *dev_args, const int64_t *dev_tile_off, int 
 {
     const ReduceArgs *args = reinterpret_cast<const ReduceArgs *>(dev_args);
     Partial *p = reinterpret_cast<Partial *>(part);
-    reduce_tiles_batch_kernel<<<(unsigned)total_tiles, kThreads, 0, s>>>(args, dev_tile_off, n_ens, p);
-    reduce_final_batch_kernel<<<n_ens, kFinalThreads, 0, s>>>(p, dev_tile_off, args, out);
+    reduce_tiles_batch_kernel<<<(unsigned)(total_tiles * kTileCtas), kThreads, 0, s>>>(
+        args, dev_tile_off, n_ens, p);
+    reduce_final_batch_kernel<<<n_ens * kFinalCtas, kThreads, 0, s>>>(p, dev_tile_off, args, out);
 }
 
 int reduce_launch(const rosen_reduce_in *in, rosen_stats *out, void *part_ws, cudaStream_t s)
@@ -350,8 +506,8 @@ int reduce_launch(const rosen_reduce_in *in, rosen_stats *out, void *part_ws, cu
     a.inv_n2 = 1.0 / ((double)in->N * (double)in->N);
     const int64_t tiles = reduce_tiles(in->C);
     Partial *part = reinterpret_cast<Partial *>(part_ws);
-    reduce_tiles_kernel<<<(unsigned)tiles, kThreads, 0, s>>>(a, part);
-    reduce_final_kernel<<<1, kFinalThreads, 0, s>>>(part, tiles, a, out);
+    reduce_tiles_kernel<<<(unsigned)(tiles * kTileCtas), kThreads, 0, s>>>(a, part);
+    reduce_final_kernel<<<kFinalCtas, kThreads, 0, s>>>(part, tiles, a, out);
     return check_launch("rosen_reduce");
 }
 
