@@ -437,6 +437,7 @@ void offlattice_make_args(const rosen_offlattice_params *p, const rosen_offlatti
     a.rf2 = (float)((1.0 + R) * (1.0 + R) * 1.001 + 1e-3);
     a.rf = (float)sqrt((double)a.rf2 * 1.0001);
     a.beta4 = lj ? (float)(4.0 * p->beta_eps) : 0.f;
+    a.six_sig2 = lj ? 6.f / a.sig2 : 0.f;
     a.dband = (float)(lj ? p->cutoff : sig * 1.001);
     if (lj) {
         const double sc = (sig * sig) / (p->cutoff * p->cutoff), s3 = sc * sc * sc;

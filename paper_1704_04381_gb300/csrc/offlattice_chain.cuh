@@ -25,6 +25,7 @@ struct OffArgs {
     int64_t C;
     float sig2, rc2, rf2, rf;  // sigma^2, cutoff^2, list radius^2 (with margin), list radius
     float beta4;               // 4 beta eps (LJ)
+    float six_sig2;            // 6 / sigma^2 (LJ)
     float dband;               // HS: sigma (the distance at which decisions flip); LJ: cutoff
     float ucut2;               // 2 |s^6 (s^6 - 1)| at the cutoff: energy jump (doubled)
     double sig2d, rc2d, beta_eps;
@@ -49,7 +50,7 @@ __host__ __device__ inline size_t chain_smem_bytes(int N, bool lj)
 
 struct ChainSmem {
     float4 *hi, *lo;   // positions (x, y, z, -)
-    float4 *nl;        // near list: g.x, g.y, g.z, 1 + |g|^2
+    float4 *nl;        // near list: g.x, g.y, g.z, 1 + |g|^2 (LJ: pairs, see put_near)
     int *nj;           // near list: bead index
     float *nb;         // near list: bound on |d^2 (FP32) - d^2 (FP64)| for this bead
     uint8_t *tr;       // chosen trial of each step
@@ -76,10 +77,39 @@ __device__ inline ChainSmem carve(unsigned char *base, int N, bool lj)
     w.hi = reinterpret_cast<float4 *>(base);
     w.lo = w.hi + N;
     w.nl = w.lo + N;
-    w.nj = reinterpret_cast<int *>(w.nl + N);
-    w.nb = reinterpret_cast<float *>(w.nj + N);
-    w.tr = reinterpret_cast<uint8_t *>(lj ? w.nb + N : w.nb);
+    w.nb = reinterpret_cast<float *>(w.nl + N);
+    w.nj = reinterpret_cast<int *>(lj ? w.nb + N : w.nb);
+    w.tr = reinterpret_cast<uint8_t *>(w.nj + N);
     return w;
+}
+
+constexpr float kNoBead = 1e30f;        // 1 + |g|^2 of no bead (beyond any u.g)
+
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+
+// Near-list entry q.  Lennard-Jones lists keep entries 2p and 2p + 1 as
+// x0 x1 y0 y1 z0 z1 c0 c1, so that the pair loop works on two beads per
+// instruction.
+template <bool LJ>
+__device__ __forceinline__ void put_near(float4 *nl, int q, const float4 &L)
+{
+    if constexpr (LJ) {
+        float *e = reinterpret_cast<float *>(nl) + (q >> 1) * 8 + (q & 1);
+        e[0] = L.x;
+        e[2] = L.y;
+        e[4] = L.z;
+        e[6] = L.w;
+    } else {
+        nl[q] = L;
+    }
+}
+
+// Approximate root: for bounds with a margin.
+__device__ __forceinline__ float root_above(float x)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
 // ---- the cell grid of long chains --------------------------------------------
@@ -397,6 +427,11 @@ struct Group {
     }
     __device__ float min(float v) const
     {
+        if constexpr (G == 32) {
+            float m;
+            asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+            return m;
+        }
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(mask, v, o, G));
         return v;
@@ -696,7 +731,7 @@ __device__ __forceinline__ int long_near_list(const OffArgs &a, const ChainLong 
             w.nls[slot] = L;
             w.njs[slot] = j;
             if (LJ) {
-                const float gn = fmaf(sqrtf(L.w - 1.f), 1.001f, 1e-6f);
+                const float gn = fmaf(root_above(L.w - 1.f), 1.001f, 1e-6f);
                 w.nbs[slot] = pair_band(gn, L.w, i - 1 - max(j, exact_upto),
                                         fminf(1.f + gn, a.dband), drift);
             }
@@ -724,7 +759,7 @@ __device__ __forceinline__ int long_near_list(const OffArgs &a, const ChainLong 
             w.nls[slot] = L;
             w.njs[slot] = j;
             if (LJ) {
-                const float gn = fmaf(sqrtf(L.w - 1.f), 1.001f, 1e-6f);
+                const float gn = fmaf(root_above(L.w - 1.f), 1.001f, 1e-6f);
                 w.nbs[slot] = pair_band(gn, L.w, i - 1 - max(j, exact_upto),
                                         fminf(1.f + gn, a.dband), drift);
             }
@@ -736,7 +771,7 @@ __device__ __forceinline__ int long_near_list(const OffArgs &a, const ChainLong 
         const int jp = w.njs[p];
         int r = 0;
         for (int t = 0; t < nn; ++t) r += w.njs[t] < jp;
-        w.nl[r] = w.nls[p];
+        put_near<LJ>(w.nl, r, w.nls[p]);
         w.nj[r] = jp;
         if (LJ) w.nb[r] = w.nbs[p];
     }
@@ -818,10 +853,10 @@ __device__ __forceinline__ void off_chain(const OffArgs &a, int64_t c, const W &
                 const unsigned m = g.vote(near);
                 if (near) {
                     const int slot = nn + __popc(m & g.below);
-                    w.nl[slot] = L;
+                    put_near<LJ>(w.nl, slot, L);
                     w.nj[slot] = j;
                     if (LJ) {
-                        const float gn = fmaf(sqrtf(L.w - 1.f), 1.001f, 1e-6f);
+                        const float gn = fmaf(root_above(L.w - 1.f), 1.001f, 1e-6f);
                         w.nb[slot] =
                             pair_band(gn, L.w, i - 1 - max(j, exact_upto),
                                       fminf(1.f + gn, a.dband), drift);
@@ -830,6 +865,10 @@ __device__ __forceinline__ void off_chain(const OffArgs &a, int64_t c, const W &
                 nn += __popc(m);
             }
             listed += (unsigned)nn;
+            if (LJ && (nn & 1) && g.gl == 0) {      // the last pair's other half
+                put_near<LJ>(w.nl, nn, make_float4(0.f, 0.f, 0.f, kNoBead));
+                w.nb[nn] = 0.f;
+            }
             __syncwarp(g.mask);
             if (!LJ && nn > 0) {
                 // One band for the step: the oldest listed bead drifted longest, and
@@ -878,25 +917,48 @@ __device__ __forceinline__ void off_chain(const OffArgs &a, int64_t c, const W &
                 Ua[s] = 0.f;
                 ncut[s] = 0;
             }
+            if constexpr (!LJ) {
 #pragma unroll 2
-            for (int q = 0; q < nn; ++q) {
-                const float4 L = w.nl[q];
-                const float bq = LJ ? w.nb[q] : 0.f;
+                for (int q = 0; q < nn; ++q) {
+                    const float4 L = w.nl[q];
 #pragma unroll
-                for (int s = 0; s < T; ++s) {
-                    const float d2 = fmaf(ux[s], L.x, fmaf(uy[s], L.y, fmaf(uz[s], L.z, L.w)));
-                    if (!LJ) {
-                        mind[s] = fminf(mind[s], d2);
-                    } else {
-                        if (d2 < a.rc2) {
-                            const float sr = __fdividef(a.sig2, d2);
-                            const float s3 = sr * sr * sr;
-                            const float e = s3 * (s3 - 1.f);
-                            U[s] += e;
-                            Ua[s] += fabsf(e);
-                            Ub[s] = fmaf(sr * s3, fabsf(2.f * s3 - 1.f) * bq, Ub[s]);
-                        }
-                        ncut[s] += fabsf(d2 - a.rc2) < bq;
+                    for (int s = 0; s < T; ++s)
+                        mind[s] = fminf(mind[s], fmaf(ux[s], L.x,
+                                                      fmaf(uy[s], L.y, fmaf(uz[s], L.z, L.w))));
+                }
+            } else {
+                // Two beads per instruction; a bead beyond the cutoff adds zeros
+                // (instead of a branch per bead).  Issue-bound; of 935 warp
+                // instructions per chain step (N = 64, k = 32) the pairs take
+                // a quarter and their error bounds a sixth.  GB300, a bead at a
+                // time before: k = 16 / 32 / 64, 5 10^5, 5 10^5, 3 10^5 chains
+                // 19.3 / 28.9 / 31.3 -> 17.5 / 26.1 / 26.7 ms; N = 150, k = 64,
+                // 3 10^4: 10.4 -> 8.6; N = 256, k = 32, 2 10^4: 12.3 -> 9.9.
+#pragma unroll 1
+                for (int q = 0; q < nn; q += 2) {
+                    const float4 xy = w.nl[q], zc = w.nl[q + 1];
+                    const float2 bq = reinterpret_cast<const float2 *>(w.nb)[q >> 1];
+#pragma unroll
+                    for (int s = 0; s < T; ++s) {
+                        const float2 d2 = __ffma2_rn(
+                            both(ux[s]), make_float2(xy.x, xy.y),
+                            __ffma2_rn(both(uy[s]), make_float2(xy.z, xy.w),
+                                       __ffma2_rn(both(uz[s]), make_float2(zc.x, zc.y),
+                                                  make_float2(zc.z, zc.w))));
+                        float2 sr = make_float2(__fdividef(a.sig2, d2.x), __fdividef(a.sig2, d2.y));
+                        if (!(d2.x < a.rc2)) sr.x = 0.f;
+                        if (!(d2.y < a.rc2)) sr.y = 0.f;
+                        const float2 s3 = __fmul2_rn(__fmul2_rn(sr, sr), sr);
+                        const float2 e = __fmul2_rn(s3, __fadd2_rn(s3, both(-1.f)));
+                        U[s] = (U[s] + e.x) + e.y;
+                        Ua[s] = (Ua[s] + fabsf(e.x)) + fabsf(e.y);
+                        const float2 z =
+                            __fmul2_rn(__fmul2_rn(__fmul2_rn(sr, s3), bq),
+                                       __ffma2_rn(both(2.f), s3, both(-1.f)));
+                        Ub[s] = (Ub[s] + fabsf(z.x)) + fabsf(z.y);
+                        const float2 f = __fadd2_rn(d2, both(-a.rc2));
+                        ncut[s] += fabsf(f.x) < bq.x;
+                        ncut[s] += fabsf(f.y) < bq.y;
                     }
                 }
             }
@@ -957,7 +1019,7 @@ __device__ __forceinline__ void off_chain(const OffArgs &a, int64_t c, const W &
                         // (Ub already carries each bead's own band.)  Trials of
                         // zero weight contribute no error (and would give 0 * inf).
                         const float dbu =
-                            a.beta4 * fmaf(6.f / a.sig2, Ub[s],
+                            a.beta4 * fmaf(a.six_sig2, Ub[s],
                                            fmaf(1e-6f, Ua[s], a.ucut2 * (float)ncut[s]));
                         if (wt[s] > 0.f)
                             err = fmaf(wt[s], dbu + fmaf(1.2e-7f, bu[s] - bmin, 3e-7f), err);
@@ -980,14 +1042,13 @@ __device__ __forceinline__ void off_chain(const OffArgs &a, int64_t c, const W &
                         P = Pn;
                     }
                     const unsigned who = g.ballot(mine >= 0);
+                    const unsigned sure = g.ballot(r - lo > E && hi - r > E);
                     if (who == 0u) {
                         ok = false;
                     } else {
                         const int src = __ffs(who) - 1;
                         sel = g.bcast(mine, src);
-                        lo = g.bcast(lo, src);
-                        hi = g.bcast(hi, src);
-                        if (!(r - lo > E) || !(hi - r > E)) ok = false;
+                        ok = (sure >> src) & 1u;
                         logS = __logf(S) - bmin;
                     }
                 }

@@ -43,7 +43,6 @@ namespace rosen {
 namespace {
 
 constexpr float kFar = 1e15f;           // coordinate of a bead not placed yet
-constexpr float kNoBead = 1e30f;        // 1 + |g|^2 of no bead (beyond any u.g)
 constexpr int kWideSelBytes = 256 * 8;  // selection table: n-th set bit of a byte
 
 // Twice the trial directions of words (a, b) and (c, d) by the special-function
@@ -77,8 +76,6 @@ __device__ __forceinline__ float min3(float a, float b, float c)
     asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
-
-__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 
 struct WideShape {
     int np;        // beads per coordinate array: N rounded up to 4 G
