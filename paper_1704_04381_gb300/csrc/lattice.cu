@@ -330,10 +330,11 @@ __global__ void __launch_bounds__(256) lattice_batch_kernel(const LatticeArgs *_
 // chain's occupied sites in an open-addressing hash table (linear probing)
 // in device memory, one 16-byte entry per 4x4x4 block of sites: the block's
 // key and a 64-bit occupancy bitmap (bit (x & 3) | (y & 3) << 2 | (z & 3) << 4).
-// A step reads only the blocks its neighbourhood touches: the end's block
-// and, per axis, the neighbouring block the neighbours (athermal, about 2.5
-// blocks per step on average) or the sites at lattice distance <= 2
-// (interacting, about 4.75) cross into -- one 16-byte load each.  Block keys
+// A step reads only the blocks its neighbourhood touches: the end's block and,
+// per axis, the neighbouring block the neighbours (athermal, about 2.5 blocks
+// per step on average) or the sites at lattice distance <= 2 (interacting,
+// about 4.75) cross into -- one 16-byte load each.  Athermal and interacting
+// chains have a kernel each (below: which differs, and why).  Block keys
 // pack 16 bits per axis; bits 48..63 of the key word hold the generation of
 // the growth that wrote it, so a lane reuses its table for the next chain
 // without clearing it (older generations read as empty).  A chain occupies at
@@ -389,7 +390,6 @@ __device__ __forceinline__ uint32_t site_bit(int qx, int qy, int qz, int dx, int
 
 // Growth number att of chain c with the sites in the lane's table tab
 // (2^logH entries).  Same rule, draws and outputs as lattice_attempt.
-template <bool kIsaw>
 __device__ __forceinline__ bool long_attempt(const LatticeArgs &a, int64_t c, uint32_t att,
                                              ulonglong2 *tab, int logH, uint32_t &gen,
                                              const uint8_t *seltab, const float *wt32,
@@ -425,15 +425,9 @@ __device__ __forceinline__ bool long_attempt(const LatticeArgs &a, int64_t c, ui
     for (int i = 1; i < N; ++i) {
         const int bx0 = ex >> 2, by0 = ey >> 2, bz0 = ez >> 2;
         const int qx = ex & 3, qy = ey & 3, qz = ez & 3;
-        // The neighbouring block per axis: athermal steps need it only when
-        // the end sits on a face of its block, interacting steps always.
+        // The neighbouring block per axis, on the side the end is nearer to.
         const int sx_ = qx <= 1 ? -1 : 1, sy_ = qy <= 1 ? -1 : 1, sz_ = qz <= 1 ? -1 : 1;
-        const bool need_x = kIsaw || qx == 0 || qx == 3;
-        const bool need_y = kIsaw || qy == 0 || qy == 3;
-        const bool need_z = kIsaw || qz == 0 || qz == 3;
         const bool fx = qx == 0 || qx == 3, fy = qy == 0 || qy == 3, fz = qz == 0 || qz == 3;
-        const bool need_xy = kIsaw && fx && fy, need_xz = kIsaw && fx && fz,
-                   need_yz = kIsaw && fy && fz;
         uint64_t want[7];
         bool need[7];
         want[0] = block_key(bx0, by0, bz0) | tag;
@@ -443,16 +437,13 @@ __device__ __forceinline__ bool long_attempt(const LatticeArgs &a, int64_t c, ui
         want[4] = block_key(bx0 + sx_, by0 + sy_, bz0) | tag;
         want[5] = block_key(bx0 + sx_, by0, bz0 + sz_) | tag;
         want[6] = block_key(bx0, by0 + sy_, bz0 + sz_) | tag;
-        need[0] = true;
-        need[1] = need_x;
-        need[2] = need_y;
-        need[3] = need_z;
-        need[4] = need_xy;
-        need[5] = need_xz;
-        need[6] = need_yz;
+        need[0] = need[1] = need[2] = need[3] = true;
+        need[4] = fx && fy;
+        need[5] = fx && fz;
+        need[6] = fy && fz;
         uint32_t h[7];
         ulonglong2 e[7];
-        constexpr int kB = kIsaw ? 7 : 4;
+        constexpr int kB = 7;
 #pragma unroll
         for (int q = 0; q < kB; ++q) {
             h[q] = block_slot(want[q] & kBlockMask, logH);
@@ -464,9 +455,7 @@ __device__ __forceinline__ bool long_attempt(const LatticeArgs &a, int64_t c, ui
             ref[q] = need[q] ? block_rest(tab, hmask, want[q], tag, h[q], e[q])
                              : BlockRef{0ull, 0u, false};
         const uint64_t b0 = ref[0].bits, bxm = ref[1].bits, bym = ref[2].bits, bzm = ref[3].bits;
-        const uint64_t bxy = kIsaw ? ref[4 < kB ? 4 : 0].bits : 0ull;
-        const uint64_t bxz = kIsaw ? ref[5 < kB ? 5 : 0].bits : 0ull;
-        const uint64_t byz = kIsaw ? ref[6 < kB ? 6 : 0].bits : 0ull;
+        const uint64_t bxy = ref[4].bits, bxz = ref[5].bits, byz = ref[6].bits;
 
         uint32_t occ = 0u, acc;
 #pragma unroll
@@ -477,7 +466,7 @@ __device__ __forceinline__ bool long_attempt(const LatticeArgs &a, int64_t c, ui
             occ |= site_bit(qx, qy, qz, ux, uy, uz, b0, bxm, bym, bzm, bxy, bxz, byz) << d;
         }
         acc = occ;
-        if (kIsaw) {
+        {
             // Contacts of neighbour d: occupied sites next to it other than
             // the end (its far site and the four beside it).
 #pragma unroll
@@ -505,7 +494,7 @@ __device__ __forceinline__ bool long_attempt(const LatticeArgs &a, int64_t c, ui
             break;
         }
         const uint32_t x = philox(make_uint4(chain, a.ens, (uint32_t)i | (att << 16), 0u), a.key).x;
-        const int sel = choose<kIsaw>(freem, m, acc, x, seltab, wt32, wt64, lw);
+        const int sel = choose<true>(freem, m, acc, x, seltab, wt32, wt64, lw);
         if (m < 4) cnt_lo += 1ull << (16 * m);
         else cnt_hi += 1ull << (16 * (m - 4));
         const int step = (sel & 1) ? -1 : 1;
@@ -556,30 +545,19 @@ __device__ __forceinline__ bool long_attempt(const LatticeArgs &a, int64_t c, ui
                 for (int q = 0; q < 3; ++q) a.coords[((int64_t)i * 3 + q) * C + c] = 0;
         return false;
     }
-    float logw;
-    if (!kIsaw) {
-        logw = 0.f;
-#pragma unroll
-        for (int q = 2; q <= 6; ++q) {
-            const uint32_t cm = (uint32_t)(((q < 4 ? cnt_lo : cnt_hi) >> (16 * (q & 3))) & 0xFFFFu);
-            logw += (float)cm * a.logm[q];
-        }
-    } else {
-        logw = lw.value();
-    }
+    const float logw = lw.value();
     if (a.logw) a.logw[c] = logw;
     if (a.r2) a.r2[c] = ex * ex + ey * ey + ez * ez;
     if (a.n2rg2) a.n2rg2[c] = (int64_t)N * sq - (sx * sx + sy * sy + sz * sz);
     return false;
 }
 
-// One lane per chain at a time, in its own table (2^logH entries at
+// One lane per interacting chain at a time, in its own table (2^logH entries at
 // ws + l 2^logH for lane l); each lane takes its next chain from the counter
 // *next as soon as it is done, so lanes whose chains die early take more.
-template <bool kIsaw>
-__global__ void __launch_bounds__(256) lattice_long_kernel(const LatticeArgs a, ulonglong2 *ws,
-                                                           int64_t lanes, int logH,
-                                                           unsigned long long *next)
+__global__ void __launch_bounds__(256) lattice_long_isaw_kernel(const LatticeArgs a, ulonglong2 *ws,
+                                                                int64_t lanes, int logH,
+                                                                unsigned long long *next)
 {
     __shared__ uint8_t seltab[kSelBytes];
     __shared__ float wt32[8];
@@ -599,7 +577,220 @@ __global__ void __launch_bounds__(256) lattice_long_kernel(const LatticeArgs a, 
         const unsigned long long c = atomicAdd(next, 1ull);
         if (c >= (unsigned long long)a.C) break;
         uint32_t att = 0;
-        while (long_attempt<kIsaw>(a, (int64_t)c, att, tab, logH, gen, seltab, wt32, wt64)) ++att;
+        while (long_attempt(a, (int64_t)c, att, tab, logH, gen, seltab, wt32, wt64)) ++att;
+    }
+}
+
+// Athermal: the end's block stays in registers, and a step looks up only the
+// one to three blocks across a face, their first probes in flight together; the
+// six neighbours are scored as the bitmap kernel for shorter chains does
+// (lattice_blocks.cuh), in 32-bit arithmetic.  Lanes step independently: one
+// whose chain ends takes the next at once instead of waiting for the warp's
+// longest.  Bound by the latency of the probes (L1 and L2 hits).  GB300, 64-bit
+// keys, a site at a time and lanes waiting for one another before, and now: N =
+// 1000, 10^6 chains 21.5 -> 18.8 ms; 4000, 5 10^4: 8.7 -> 6.5; 10^4, 2 10^5:
+// 44 -> 27.  (Interacting chains, with six look-ups a step, lose what they
+// gain: N = 1000, 2 10^5 chains, beta eps = 0.3, 7.3 ms before, 8.0 this way.)
+constexpr uint32_t kMulXY = 0x9E3779B1u, kMulZ = 0x85EBCA77u;   // hash of (x | y << 16, z)
+
+struct LongWalk {
+    int ex, ey, ez;
+    int sx, sy, sz;            // |sum| <= N^2 / 2 < 2^30
+    int64_t sq;
+    uint64_t cnt_lo, cnt_hi;   // 16-bit fields: m = 0..3 | 4..7
+    int p;                     // the end's place in its block: x + 4 y + 16 z
+    uint32_t xy, zg;           // the block: x | y << 16, z | generation << 16
+    uint32_t h;                // its entry
+    uint2 cur;                 // and its bitmap
+};
+
+__device__ __forceinline__ void begin_long(LongWalk &w, uint4 *tab, int logH, uint32_t &gen)
+{
+    if (++gen > kGenMax) {          // generation tags exhausted: clear the table
+        for (uint32_t h = 0; h < (1u << logH); ++h) tab[h] = make_uint4(0u, 0u, 0u, 0u);
+        gen = 1;
+    }
+    w.ex = w.ey = w.ez = w.sx = w.sy = w.sz = 0;
+    w.sq = 0;
+    w.cnt_lo = w.cnt_hi = 0ull;
+    w.p = 0;
+    w.xy = 0x80008000u;             // block (0, 0, 0), biased by 32768 per axis
+    w.zg = 0x8000u | (gen << 16);
+    w.cur = make_uint2(1u, 0u);     // site (0, 0, 0): bit 0
+    w.h = (w.xy * kMulXY + 0x8000u * kMulZ) >> (32 - logH);
+    tab[w.h] = make_uint4(w.xy, w.zg, w.cur.x, w.cur.y);
+}
+
+// One step with draw x: the number of free neighbours (0: trapped); sel: the
+// neighbour taken.
+__device__ __forceinline__ int step_long(LongWalk &w, uint4 *tab, int logH, uint32_t gen, uint32_t x,
+                                         const uint8_t *seltab, const uint2 *masks, int &sel)
+{
+    constexpr int K = kSiteBlocks<false>;
+    const uint32_t hmask = (1u << logH) - 1u;
+    const int p = w.p, qx = p & 3, qy = (p >> 2) & 3, qz = p >> 4;
+    const uint32_t cx = (0x42u >> (2 * qx)) & 3u, cy = (0x42u >> (2 * qy)) & 3u,
+                   cz = (0x42u >> (2 * qz)) & 3u;
+    const uint32_t across = cx | (cy << 2) | (cz << 4);
+    const uint32_t ox = qx > 1 ? 1u : 0xFFFFFFFFu, oy = qy > 1 ? 0x10000u : 0xFFFF0000u,
+                   oz = qz > 1 ? 1u : 0xFFFFFFFFu;
+    uint32_t xy[K], zg[K], h[K];
+    bool need[K];
+    xy[0] = w.xy + ox;
+    xy[1] = w.xy + oy;
+    xy[2] = w.xy;
+    zg[0] = zg[1] = w.zg;
+    zg[2] = w.zg + oz;
+    need[0] = cx;
+    need[1] = cy;
+    need[2] = cz;
+    uint4 e[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        h[q] = (xy[q] * kMulXY + (zg[q] & 0xFFFFu) * kMulZ) >> (32 - logH);
+        e[q] = need[q] ? tab[h[q]] : make_uint4(0u, 0u, 0u, 0u);
+    }
+    uint2 nb[K];
+    bool found[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        while ((e[q].y >> 16) == gen && !(e[q].x == xy[q] && e[q].y == zg[q])) {
+            h[q] = (h[q] + 1u) & hmask;
+            e[q] = tab[h[q]];
+        }
+        found[q] = (e[q].y >> 16) == gen;
+        nb[q] = found[q] ? make_uint2(e[q].z, e[q].w) : make_uint2(0u, 0u);
+    }
+    const uint32_t acc = sites_around<false>(p, w.cur, nb, masks);
+    const uint32_t freem = ~acc & 63u;
+    const int m = __popc(freem);
+    if (m == 0) return 0;
+    LogW none;
+    sel = choose<false>(freem, m, acc, x, seltab, nullptr, nullptr, none);
+    if (m < 4) w.cnt_lo += 1ull << (16 * m);
+    else w.cnt_hi += 1ull << (16 * (m - 4));
+
+    // The new site, in the end's block or across a face.
+    const int axis2 = sel & 6, s = 1 << axis2;
+    const int dir = (sel & 1) ? -1 : 1;
+    if ((across >> sel) & 1u) {
+        const bool first = axis2 == 0, second = axis2 == 2;
+        const bool old = first ? found[0] : (second ? found[1] : found[2]);
+        w.cur.x = first ? nb[0].x : (second ? nb[1].x : nb[2].x);
+        w.cur.y = first ? nb[0].y : (second ? nb[1].y : nb[2].y);
+        w.h = first ? h[0] : (second ? h[1] : h[2]);
+        w.xy = first ? xy[0] : (second ? xy[1] : xy[2]);
+        w.zg = first ? zg[0] : (second ? zg[1] : zg[2]);
+        w.p = p - 3 * dir * s;
+        if (!old) reinterpret_cast<uint2 *>(tab + w.h)[0] = make_uint2(w.xy, w.zg);
+    } else {
+        w.p = p + dir * s;
+    }
+    if (w.p & 32) w.cur.y |= 1u << (w.p & 31);
+    else w.cur.x |= 1u << (w.p & 31);
+    reinterpret_cast<uint2 *>(tab + w.h)[1] = w.cur;
+    if (axis2 == 0) w.ex += dir;
+    else if (axis2 == 2) w.ey += dir;
+    else w.ez += dir;
+    w.sx += w.ex;
+    w.sy += w.ey;
+    w.sz += w.ez;
+    w.sq += (int64_t)w.ex * w.ex + (int64_t)w.ey * w.ey + (int64_t)w.ez * w.ez;
+    return m;
+}
+
+// Outputs of a finished chain (dead: trapped at step i).
+__device__ __forceinline__ void finish_long(const LatticeArgs &a, int64_t c, uint32_t att, int i,
+                                            bool dead, LongWalk &w)
+{
+    const int N = a.N;
+    const int64_t C = a.C;
+    if (a.attempts) a.attempts[c] = (uint16_t)(att + 1);
+    if (dead) w.cnt_lo += 1ull;   // counts[0] = 1 marks the dead end
+    if (a.counts)
+        a.counts[c] = make_uint4((uint32_t)w.cnt_lo, (uint32_t)(w.cnt_lo >> 32), (uint32_t)w.cnt_hi,
+                                 (uint32_t)(w.cnt_hi >> 32));
+    float logw = dead ? -INFINITY : 0.f;
+    if (!dead)
+#pragma unroll
+        for (int q = 2; q <= 6; ++q) {
+            const uint32_t cm = (uint32_t)(((q < 4 ? w.cnt_lo : w.cnt_hi) >> (16 * (q & 3))) & 0xFFFFu);
+            logw += (float)cm * a.logm[q];
+        }
+    if (a.logw) a.logw[c] = logw;
+    if (a.r2) a.r2[c] = dead ? 0 : w.ex * w.ex + w.ey * w.ey + w.ez * w.ez;
+    if (a.n2rg2)
+        a.n2rg2[c] = dead ? 0
+                          : (int64_t)N * w.sq - ((int64_t)w.sx * w.sx + (int64_t)w.sy * w.sy +
+                                                 (int64_t)w.sz * w.sz);
+    if (dead) {
+        if (a.trace) {
+            a.trace[(int64_t)(i - 1) * C + c] = 7u;
+            for (int s = i + 1; s < N; ++s) a.trace[(int64_t)(s - 1) * C + c] = 0xFFu;
+        }
+        if (a.coords)
+            for (int s = 3 * i; s < 3 * N; ++s) a.coords[(int64_t)s * C + c] = 0;
+    }
+}
+
+// Lane l of the grid works in its own table (2^logH entries at ws + l 2^logH)
+// and takes its chains from the counter *next.
+__global__ void __launch_bounds__(256) lattice_long_kernel(const LatticeArgs a, uint4 *ws,
+                                                           int64_t lanes, int logH,
+                                                           unsigned long long *next)
+{
+    __shared__ uint8_t seltab[kSelBytes];
+    __shared__ uint2 masks[12];
+    fill_site_masks(masks);
+    for (int q = threadIdx.x; q < kSelBytes; q += blockDim.x)
+        seltab[q] = nth_set_bit((uint32_t)q >> 3, (uint32_t)q & 7u);
+    __syncthreads();
+    const int64_t lane = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    bool more = lane < lanes;
+    uint4 *const tab = ws + ((more ? lane : 0) << logH);
+    uint32_t gen = 0u, att = 0u;
+    int64_t c = -1;
+    int i = 0;
+    LongWalk w;
+    for (;;) {
+        if (c < 0 && more) {
+            const unsigned long long n = atomicAdd(next, 1ull);
+            more = n < (unsigned long long)a.C;
+            if (more) {
+                c = (int64_t)n;
+                att = 0u;
+                i = 1;
+                begin_long(w, tab, logH, gen);
+                first_monomer(a, c);
+            }
+        }
+        if (!__any_sync(0xffffffffu, c >= 0)) break;
+        if (c >= 0) {
+            const uint32_t x = philox(make_uint4(a.chain0 + (uint32_t)c, a.ens,
+                                                 (uint32_t)i | (att << 16), 0u), a.key).x;
+            int sel = 0;
+            const int m = step_long(w, tab, logH, gen, x, seltab, masks, sel);
+            if (m > 0) {
+                if (a.trace) a.trace[(int64_t)(i - 1) * a.C + c] = (uint8_t)((m << 3) | sel);
+                if (a.coords) {
+                    a.coords[((int64_t)i * 3 + 0) * a.C + c] = w.ex;
+                    a.coords[((int64_t)i * 3 + 1) * a.C + c] = w.ey;
+                    a.coords[((int64_t)i * 3 + 2) * a.C + c] = w.ez;
+                }
+                if (++i == a.N) {
+                    finish_long(a, c, att, i, false, w);
+                    c = -1;
+                }
+            } else if (att + 1 < a.max_att) {
+                ++att;
+                i = 1;
+                begin_long(w, tab, logH, gen);
+            } else {
+                finish_long(a, c, att, i, true, w);
+                c = -1;
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -846,7 +1037,7 @@ extern "C" size_t rosen_lattice_long_workspace_size(int32_t N, int64_t C)
 {
     if (N < 2 || N > ROSEN_LATTICE_LONG_NMAX || C < 1) return 0;
     const int64_t lanes = C < kLongLanes ? C : kLongLanes;
-    return kLongHeader + (size_t)lanes * (sizeof(ulonglong2) << long_log_entries(N));
+    return kLongHeader + (size_t)lanes * (sizeof(uint4) << long_log_entries(N));
 }
 
 extern "C" int rosen_lattice_grow_long(const rosen_lattice_params *p, const rosen_lattice_out *o,
@@ -859,7 +1050,7 @@ extern "C" int rosen_lattice_grow_long(const rosen_lattice_params *p, const rose
         return set_error(ROSEN_EINVAL, "rosen_lattice_grow_long: workspace must be a non-NULL, "
                                        "16-byte aligned device pointer");
     const int logH = long_log_entries(p->N);
-    const size_t table = sizeof(ulonglong2) << logH;
+    const size_t table = sizeof(uint4) << logH;
     int64_t lanes = workspace_bytes > kLongHeader
                         ? (int64_t)((workspace_bytes - kLongHeader) / table) : 0;
     if (lanes > p->C) lanes = p->C;
@@ -877,10 +1068,12 @@ extern "C" int rosen_lattice_grow_long(const rosen_lattice_params *p, const rose
                          (long long)lanes, table, cudaGetErrorString(e));
     const unsigned grid = (unsigned)((lanes + 255) / 256);
     unsigned long long *next = static_cast<unsigned long long *>(workspace);
-    ulonglong2 *ws = reinterpret_cast<ulonglong2 *>(static_cast<unsigned char *>(workspace) +
-                                                    kLongHeader);
-    if (a.isaw) lattice_long_kernel<true><<<grid, 256, 0, s>>>(a, ws, lanes, logH, next);
-    else lattice_long_kernel<false><<<grid, 256, 0, s>>>(a, ws, lanes, logH, next);
+    unsigned char *ws = static_cast<unsigned char *>(workspace) + kLongHeader;
+    if (a.isaw)
+        lattice_long_isaw_kernel<<<grid, 256, 0, s>>>(a, reinterpret_cast<ulonglong2 *>(ws), lanes,
+                                                      logH, next);
+    else
+        lattice_long_kernel<<<grid, 256, 0, s>>>(a, reinterpret_cast<uint4 *>(ws), lanes, logH, next);
     return check_launch("rosen_lattice_grow_long (kernel launch)");
 }
 

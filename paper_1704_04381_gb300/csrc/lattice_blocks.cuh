@@ -161,55 +161,32 @@ __device__ __forceinline__ void begin_sites(SiteWalk &w, const SiteTable &t)
     t.bits[w.h * t.step] = w.cur;
 }
 
-// One step from the chain's end with draw x.  Returns the number of free
-// neighbours (0: trapped), -1 if the table is full; sel: the neighbour taken.
+// Blocks a step looks up: across the face the end is nearer to on x, y and z;
+// interacting chains also across two faces (x y, x z, y z).
 template <bool kIsaw>
-__device__ __forceinline__ int step_sites(SiteWalk &w, const SiteTable &t, uint32_t x,
-                                          const uint8_t *seltab, const uint2 *masks,
-                                          const float *wt32, const double *wt64, int &sel)
-{
-    const int p = w.p, qx = p & 3, qy = (p >> 2) & 3, qz = p >> 4;
-    // Two bits per axis, + and -: the neighbour lies across a face.
-    const uint32_t cx = (0x42u >> (2 * qx)) & 3u, cy = (0x42u >> (2 * qy)) & 3u,
-                   cz = (0x42u >> (2 * qz)) & 3u;
-    const uint32_t across = cx | (cy << 2) | (cz << 4);
-    // The neighbouring block per axis lies on the side the end is nearer to:
-    // sites within two steps reach no other.
-    const uint32_t ox = qx > 1 ? 1u : 0xFFFFFFFFu, oy = qy > 1 ? 256u : 0xFFFFFF00u,
-                   oz = qz > 1 ? 65536u : 0xFFFF0000u;
-    const int tx = qx > 1 ? p - 4 : p + 4, ty = qy > 1 ? p - 16 : p + 16;
-    constexpr int K = kIsaw ? 6 : 3;
-    uint32_t want[K];
-    bool need[K];
-    want[0] = w.key + ox;
-    want[1] = w.key + oy;
-    want[2] = w.key + oz;
-    need[0] = kIsaw || cx;
-    need[1] = kIsaw || cy;
-    need[2] = kIsaw || cz;
-    if constexpr (kIsaw) {
-        // Blocks across two faces: x y, x z, y z.
-        want[3] = want[0] + oy;
-        want[4] = want[0] + oz;
-        want[5] = want[1] + oz;
-        need[3] = cx && cy;
-        need[4] = cx && cz;
-        need[5] = cy && cz;
-    }
-    SiteRef ref[K];
-    find_sites<K>(t, want, need, ref);
+constexpr int kSiteBlocks = kIsaw ? 6 : 3;
 
+// What lies around the end at place p of its block (bitmap cur), nb[] the
+// bitmaps of the neighbouring blocks: bits 0..5, neighbour d is occupied; bits
+// 8+3d..10+3d (interacting), the contacts of neighbour d.
+template <bool kIsaw>
+__device__ __forceinline__ uint32_t sites_around(int p, uint2 cur,
+                                                 const uint2 (&nb)[kSiteBlocks<kIsaw>],
+                                                 const uint2 *masks)
+{
+    const int qx = p & 3, qy = (p >> 2) & 3, qz = p >> 4;
+    const int tx = qx > 1 ? p - 4 : p + 4, ty = qy > 1 ? p - 16 : p + 16;
     // The sites around the end in one turned bitmap: those of the end's block,
     // those across a face from its neighbours' bitmaps, turned to match.
     const uint2 mx = masks[qx], my = masks[4 + qy], mz = masks[8 + qz];
-    uint2 M = turn(w.cur, p);
-    const uint2 X = turn(ref[0].bits, tx), Y = turn(ref[1].bits, ty), Z = turn(ref[2].bits, p);
+    uint2 M = turn(cur, p);
+    const uint2 X = turn(nb[0], tx), Y = turn(nb[1], ty), Z = turn(nb[2], p);
     uint32_t two_in = 0u, two_out = 0u;    // two steps along z, in the block and across
     if constexpr (kIsaw) {
         two_in = M.y & 1u;
         two_out = Z.y & 1u;
-        const uint2 XY = turn(ref[3].bits, qy > 1 ? tx - 16 : tx + 16), XZ = turn(ref[4].bits, tx),
-                    YZ = turn(ref[5].bits, ty);
+        const uint2 XY = turn(nb[3], qy > 1 ? tx - 16 : tx + 16), XZ = turn(nb[4], tx),
+                    YZ = turn(nb[5], ty);
         M = mix(mix(M, X, mx), mix(Y, XY, mx), my);
         M = mix(M, mix(mix(Z, XZ, mx), YZ, my), mz);
     } else {
@@ -234,6 +211,50 @@ __device__ __forceinline__ int step_sites(SiteWalk &w, const SiteTable &t, uint3
             acc |= cd << (8 + 3 * d);
         }
     }
+    return acc;
+}
+
+// One step from the chain's end with draw x.  Returns the number of free
+// neighbours (0: trapped), -1 if the table is full; sel: the neighbour taken.
+template <bool kIsaw>
+__device__ __forceinline__ int step_sites(SiteWalk &w, const SiteTable &t, uint32_t x,
+                                          const uint8_t *seltab, const uint2 *masks,
+                                          const float *wt32, const double *wt64, int &sel)
+{
+    const int p = w.p, qx = p & 3, qy = (p >> 2) & 3, qz = p >> 4;
+    // Two bits per axis, + and -: the neighbour lies across a face.
+    const uint32_t cx = (0x42u >> (2 * qx)) & 3u, cy = (0x42u >> (2 * qy)) & 3u,
+                   cz = (0x42u >> (2 * qz)) & 3u;
+    const uint32_t across = cx | (cy << 2) | (cz << 4);
+    // The neighbouring block per axis lies on the side the end is nearer to:
+    // sites within two steps reach no other.
+    const uint32_t ox = qx > 1 ? 1u : 0xFFFFFFFFu, oy = qy > 1 ? 256u : 0xFFFFFF00u,
+                   oz = qz > 1 ? 65536u : 0xFFFF0000u;
+    constexpr int K = kSiteBlocks<kIsaw>;
+    uint32_t want[K];
+    bool need[K];
+    want[0] = w.key + ox;
+    want[1] = w.key + oy;
+    want[2] = w.key + oz;
+    need[0] = kIsaw || cx;
+    need[1] = kIsaw || cy;
+    need[2] = kIsaw || cz;
+    if constexpr (kIsaw) {
+        // Blocks across two faces: x y, x z, y z.
+        want[3] = want[0] + oy;
+        want[4] = want[0] + oz;
+        want[5] = want[1] + oz;
+        need[3] = cx && cy;
+        need[4] = cx && cz;
+        need[5] = cy && cz;
+    }
+    SiteRef ref[K];
+    find_sites<K>(t, want, need, ref);
+
+    uint2 nb[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) nb[q] = ref[q].bits;
+    const uint32_t acc = sites_around<kIsaw>(p, w.cur, nb, masks), occ = acc & 63u;
     const uint32_t freem = ~occ & 63u;
     const int m = __popc(freem);
     if (m == 0) return 0;
