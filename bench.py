@@ -52,11 +52,10 @@ BRUTE_LAT_PAIR, BRUTE_LAT_STEP = 7, 100
 BRUTE_OFF_PAIR, BRUTE_OFF_TRIAL = 8, 90
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
-# the dominant growth -- hard spheres, N = 64, k = 32, 10^7 chains, both
-# passes -- from one ncu capture of that launch: first pass 23,213,312 +
-# 78,660,864, second pass 18,835,968 + 17,702,912.  Reported as the
-# roofline's traffic for that configuration only.
-HS_TRAFFIC_BYTES = 22961664 + 78489856 + 18875648 + 18076160
+# the dominant growth -- hard spheres, N = 64, k = 32, 10^7 chains -- from one
+# ncu capture of that launch.  Reported as the roofline's traffic for that
+# configuration only.
+HS_TRAFFIC_BYTES = 2774016 + 76424704
 
 
 def brute_lattice_ops(N):
@@ -389,14 +388,15 @@ def run_ours(args):
         "data": "synthetic (Philox-seeded growth; no input data)",
         "config": step_config(world, args.max_attempts),
         "parts": parts,
-        "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12,
-                     "unit": "Tops/s (32-bit lane ops)", "frac": achieved / peak,
+        "roofline": {"bound": "alu", "achieved": executed / 1e12, "peak": peak / 1e12,
+                     "unit": "Tops/s (32-bit lane ops)", "frac": executed / peak,
                      "traffic": (HS_TRAFFIC_BYTES if (REAL_POT == "hard_sphere" and C == 10_000_000
                                                       and K_TRIALS == 32 and args.max_attempts <= 1
-                                                      and "hard sphere" in kname) else None),
-                     "traffic_unit": "DRAM bytes per launch (ncu, both passes)",
-                     "kernel": kname, "ops_per_chain": sops / C,
-                     "ops_basis": "brute-force work: every earlier monomer tested against every trial",
+                                                      and "wide" in kname) else None),
+                     "traffic_unit": "DRAM bytes per launch (ncu)",
+                     "kernel": kname, "ops_per_chain": ops / C,
+                     "ops_basis": "operations made: beads scanned, near beads tested, trials drawn",
+                     "brute_ops_per_chain": sops / C, "brute_frac": achieved / peak,
                      "executed_ops_per_chain": ops / C, "executed_frac": executed / peak,
                      "peak_basis": "%d SMs x 128 lanes x %.0f MHz (max SM clock)" % (sms, mhz)},
         "clocks": clocks.summary(),

@@ -186,7 +186,11 @@ typedef struct rosen_offlattice_params {
     double beta_eps;          /* LJ well depth over kT, >= 0, finite        */
     uint32_t flags;           /* ROSEN_STORE_TRACE | ROSEN_STORE_COORDS     */
     int32_t lanes_per_chain;  /* 0 = automatic; else 8, 16 or 32 lanes grow
-                                 one chain (k <= 4 * lanes_per_chain)       */
+                                 one chain (k <= 4 * lanes_per_chain).  Hard
+                                 spheres in rosen_offlattice_grow: the kernel
+                                 picks its lanes; the value sets the order of
+                                 the R_g^2 sum, so that results equal those
+                                 of the other entry points with these lanes */
     int32_t max_attempts;     /* 0 or 1: a dead end keeps W = 0.  2 ..
                                  ROSEN_MAX_ATTEMPTS: restart mode (Section
                                  3.3.3): the chain is grown again from bead
