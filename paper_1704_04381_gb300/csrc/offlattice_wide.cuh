@@ -20,19 +20,20 @@
 //     arithmetic works on pairs of trials (two results per instruction);
 //  4. selection; a step the fast directions cannot decide within their error
 //     band is decided again by the whole warp (wide_redecide);
-//  5. commit of the chosen trial's direction, taken again as off_chain does.
+//  5. commit of the chosen trial's direction, taken again as off_chain does
+//     from the words its lane kept.
 // Displacements, bands, draws, sums and the steps re-decided in FP64 are those
 // of off_chain with Gref lanes per chain, operation for operation: a chain's
 // outputs are the same bit for bit.  (The order of a hard-sphere list does
 // not matter: a minimum.)
 //
-// It is bound by issue (64%) with 16 warps per SM, the most 128 registers and
-// 24 bytes a bead leave: 119 warp instructions per chain step.  GB300, before
+// It is bound by issue (65%) with 16 warps per SM, the most 128 registers and
+// 24 bytes a bead leave: 118 warp instructions per chain step.  GB300, before
 // (16 or 32 lanes, FP64 re-decision in a second pass or in place) and now, k =
-// 32: N = 64, 10^7 chains 171 -> 94 ms; N = 128, 2 10^5: 11.3 -> 5.8; N = 256,
-// 6 10^4: 10.4 -> 5.8; N = 512, 2 10^4: 17.7 -> 6.7; N = 1024, 5 10^3: 18.5 ->
-// 5.8.  N = 64: k = 16, 5 10^5 chains 7.9 -> 4.2; k = 64, 3 10^5: 8.3 -> 5.2;
-// k = 128, 2 10^5: 9.6 -> 6.4; k = 32, 100 chains 0.23 -> 0.13.  Tried and not kept: all trials
+// 32: N = 64, 10^7 chains 171 -> 91 ms; N = 128, 2 10^5: 11.3 -> 5.8; N = 256,
+// 6 10^4: 10.4 -> 5.5; N = 512, 2 10^4: 17.7 -> 6.3; N = 1024, 5 10^3: 18.5 ->
+// 5.4.  N = 64: k = 16, 5 10^5 chains 7.9 -> 3.7; k = 64, 3 10^5: 8.3 -> 5.0;
+// k = 128, 2 10^5: 9.6 -> 6.2; k = 32, 100 chains 0.23 -> 0.12.  Tried and not kept: all trials
 // through dir32x2 (13.5 ms), per-chain lists ranked by votes (12.5), the next
 // step's trials drawn beside the selection (11.4: more registers moved).
 #pragma once
@@ -517,6 +518,7 @@ __global__ void __launch_bounds__(512, 1) offlattice_wide_kernel(const __grid_co
 
         // ---- 2. trials -------------------------------------------------------------------
         float2 ux[T / 2], uy[T / 2], uz[T / 2];      // 2u: d^2 = c + (2u).g
+        uint4 words[T / 2];
         float mind[T];
         uint32_t selw = 0u;
 #pragma unroll
@@ -526,6 +528,7 @@ __global__ void __launch_bounds__(512, 1) offlattice_wide_kernel(const __grid_co
             if (s == 0)
                 selw = __byte_perm(__byte_perm(x.x, x.y, 0x0040u), __byte_perm(x.z, x.w, 0x0040u),
                                    0x5410u);
+            words[s] = x;
             fast_dirs_x2(x, ux[s], uy[s], uz[s]);
             mind[2 * s] = mind[2 * s + 1] = INFINITY;
         }
@@ -615,7 +618,17 @@ __global__ void __launch_bounds__(512, 1) offlattice_wide_kernel(const __grid_co
         const bool mine = r >= 0 && r < cnt;
         const int ss = nth[(fr << 3) | (uint32_t)(mine ? r : 0)];
         const unsigned who = __ballot_sync(kAll, mine) & g.mask;
-        int sel = __shfl_sync(kAll, T * g.gl + ss, who ? __ffs(who) - 1 : g.base);
+        const int src = who ? __ffs(who) - 1 : g.base;
+        int sel = __shfl_sync(kAll, T * g.gl + ss, src);
+        // Its Philox words, kept since the trials were drawn: T selects and two
+        // shuffles in place of a ten-round call by every lane (N = 64, k = 32,
+        // 10^6 chains: 9.57 -> 9.26 ms, no more registers).
+        uint32_t ca = words[0].x, cb = words[0].y;
+#pragma unroll
+        for (int s = 0; s < T; ++s)
+            if (s == ss) trial_words(words[s / 2], s, ca, cb);
+        ca = __shfl_sync(kAll, ca, src);
+        cb = __shfl_sync(kAll, cb, src);
 
         // Steps FP32 cannot decide, a chain at a time with the whole warp.
         unsigned amb = __ballot_sync(kAll, on && flag);
@@ -634,7 +647,12 @@ __global__ void __launch_bounds__(512, 1) offlattice_wide_kernel(const __grid_co
                 ely = d.ly;
                 elz = d.lz;
                 m = d.m;
-                sel = d.sel;
+                if (sel != d.sel) {
+                    sel = d.sel;
+                    const uint4 xs =
+                        philox(make_uint4(chain, a.ens, step, 1u + (uint32_t)(sel >> 1)), a.key);
+                    trial_words(xs, sel, ca, cb);
+                }
                 if (d.exact) {
                     exact_upto = i - 1;
                     ++rechecks;
@@ -643,10 +661,7 @@ __global__ void __launch_bounds__(512, 1) offlattice_wide_kernel(const __grid_co
         }
 
         // ---- 5. commit: the chosen trial's direction, exactly as off_chain ------------
-        const uint4 xs = philox(make_uint4(chain, a.ens, step, 1u + (uint32_t)(sel >> 1)), a.key);
-        uint32_t wa, wb;
-        trial_words(xs, sel, wa, wb);
-        const float3 u2 = dir32x2(wa, wb);
+        const float3 u2 = dir32x2(ca, cb);
         const bool dead = m == 0;
         if (on && !dead) {
             if (g.gl == 0) {
