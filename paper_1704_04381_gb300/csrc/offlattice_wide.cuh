@@ -414,6 +414,7 @@ __global__ void __launch_bounds__(512, 1) offlattice_wide_kernel(const __grid_co
     float4 *const near = reinterpret_cast<float4 *>(P + 6 * np);   // a near bead per lane
     uint8_t *const tr = reinterpret_cast<uint8_t *>(P + 6 * np + 8 * G);
     for (int q = g.gl; q < sh.stride; q += G) P[q] = 0.f;   // (what is read is finite)
+    __syncwarp();                         // before restart() writes the same words from other lanes
     const int N = a.N, k = a.k;
     const auto put = [&](int j, float hx, float hy, float hz, float lx, float ly, float lz) {
         const int p = wide_at<G>(j);
