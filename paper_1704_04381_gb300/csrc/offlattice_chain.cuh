@@ -429,7 +429,7 @@ struct Group {
     {
         if constexpr (G == 32) {
             float m;
-            asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+            asm volatile("redux.sync.min.f32 %0, %1, %2;" : "=f"(m) : "f"(v), "r"(mask));
             return m;
         }
 #pragma unroll
