@@ -284,6 +284,14 @@ ROSEN_API int rosen_offlattice_grow_long(const rosen_offlattice_params *p,
 ROSEN_API int rosen_sphere_points(const uint32_t *words, int64_t n, float *out, void *stream);
 
 /*
+ * The same unit vectors by the special-function unit, as the hard-sphere kernel
+ * tests its trials (the chosen one is taken again as above).  out: device, 3n
+ * floats.  Exposed so that the bound on the difference of the two can be checked
+ * exhaustively.
+ */
+ROSEN_API int rosen_sphere_points_fast(const uint32_t *words, int64_t n, float *out, void *stream);
+
+/*
  * The same unit vectors as float-float components, as the Lennard-Jones
  * kernels add them to the chain's position (no paper counterpart: it keeps
  * positions within ~1e-12 per step of exact).  out: device, 5n floats per

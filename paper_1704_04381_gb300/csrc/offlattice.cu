@@ -147,6 +147,20 @@ __global__ void sphere_points_kernel(const uint2 *words, int64_t n, float *out)
     out[3 * q + 2] = u.z;
 }
 
+// The hard-sphere kernel's fast directions (twice the unit vectors; halving is
+// exact).
+__global__ void sphere_points_fast_kernel(const uint2 *words, int64_t n, float *out)
+{
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const uint2 v = words[q];
+    float2 x, y, z;
+    fast_dirs_x2(make_uint4(v.x, v.y, v.x, v.y), x, y, z);
+    out[3 * q + 0] = 0.5f * x.x;
+    out[3 * q + 1] = 0.5f * y.x;
+    out[3 * q + 2] = 0.5f * z.x;
+}
+
 // Float-float directions as the Lennard-Jones kernels commit them.
 __global__ void sphere_points_ff_kernel(const uint2 *words, int64_t n, float *out)
 {
@@ -566,6 +580,20 @@ extern "C" int rosen_sphere_points(const uint32_t *words, int64_t n, float *out,
     sphere_points_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0,
                            (cudaStream_t)stream>>>(reinterpret_cast<const uint2 *>(words), n, out);
     return check_launch("rosen_sphere_points");
+}
+
+extern "C" int rosen_sphere_points_fast(const uint32_t *words, int64_t n, float *out, void *stream)
+{
+    if (n < 0) return set_error(ROSEN_EINVAL, "rosen_sphere_points_fast: n < 0");
+    if (n > 0 && (!words || !out)) return set_error(ROSEN_EINVAL, "rosen_sphere_points_fast: NULL");
+    if (reinterpret_cast<uintptr_t>(words) & 7u)
+        return set_error(ROSEN_EINVAL, "rosen_sphere_points_fast: words must be 8-byte aligned");
+    if (n == 0) return ROSEN_OK;
+    const int threads = 256;
+    sphere_points_fast_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0,
+                                (cudaStream_t)stream>>>(reinterpret_cast<const uint2 *>(words), n,
+                                                        out);
+    return check_launch("rosen_sphere_points_fast");
 }
 
 extern "C" int rosen_sphere_points_ff(const uint32_t *words, int64_t n, float *out, void *stream)

@@ -48,12 +48,22 @@ constexpr int kWideSelBytes = 256 * 8;  // selection table: n-th set bit of a by
 
 // Twice the trial directions of words (a, b) and (c, d) by the special-function
 // unit, as pairs: the angle in (-pi, pi] from the signed word, sin, cos and
-// sqrt approximate.  Over all 2^24 angles and all 2^24 polar words a direction
-// is within 3.7e-7 (angle) + 7.4e-8 (s) of exact, and dir32x2 / 2 within
-// 2.7e-7, so a squared distance d^2 = c + 2 u.g moves by at most
-// 2 (4.4e-7 + 2.7e-7) |g| when one takes the place of the other: kFastBand |g|
-// on top of the band.  The chosen trial's direction is taken again with dir32x2.
-constexpr float kFastBand = 1.6e-6f;
+// sqrt approximate.  The chosen trial's direction is taken again with dir32x2.
+// As vectors (Euclidean norm) the two differ by less than kFastDir: 7.6e-7 over
+// all 2^24 angles at s = 1, 1.2e-7 over all 2^24 polar words at angle 0, and at
+// most 1.7e-7 by the rounding of both sides' products with s; z is the same.
+// (Largest difference of 2^31 random directions: 9.1e-7.)
+constexpr double kFastDir = 1.06e-6;
+
+// What a squared distance d^2 = c + 2u.g at the decision (d^2 <= sigma^2 + 0.01,
+// |g| < rf) differs by between fast_dirs_x2 and dir32x2: kFastDir |g|, and on
+// either side the rounding of c + 2 uz gz, of that + 2 uy gy and of d^2, which
+// are at most d^2 + 2^(3/2) |g|, d^2 + 2 |g| and d^2.  Together below kFastBand rf,
+// as rf > 1 + sigma and sigma <= 4 (sigma^2 / rf < 3.2).  A step whose fast
+// distances stay out of pair_band plus this is one that off_chain decides in
+// FP32, and alike.  (N = 64, k = 32: a band three times as wide costs 0.1%.)
+constexpr float kFastBand = 2.8e-6f;
+static_assert(kFastBand > kFastDir + 2.0 * 0x1p-24 * (3.0 * (3.2 + 0.01) + 4.83), "fast band");
 
 __device__ __forceinline__ void fast_dirs_x2(const uint4 &w, float2 &x, float2 &y, float2 &z)
 {
