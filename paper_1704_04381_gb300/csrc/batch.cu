@@ -9,15 +9,18 @@
 // ensembles share the GPU without tail effects.  The shape of every class
 // (lattice: chains per block; real space: lanes per chain) is picked by timing
 // the candidates on a sample of the class.  A member with at least
-// kOwnLaunchWaves times the chains its single-ensemble kernel grows at once
+// own_launch_waves() times the chains its single-ensemble kernel grows at once
 // fills the GPU by itself: it runs as that kernel's own launch (a persistent
 // grid over its chains) on the class's stream, before the class kernel, and
 // the class kernel serves the smaller members.  Growth of all classes (on
 // forked streams, so they overlap) and the FP64 reduction of every ensemble
 // are captured once into a CUDA graph; each run is one graph launch.
 //
-// Every chain is grown by the same device code as the single-ensemble entry
-// points and every ensemble is reduced by the same tile and merge code as
+// The class kernels grow a chain with the rule, draws and arithmetic of the
+// single-ensemble entry points (Lennard-Jones and lattice chains below N = 160
+// with the same device code; hard spheres with off_chain and longer lattice
+// chains with the key scan, whose outputs the few-lanes and bitmap kernels equal
+// bit for bit), and every ensemble is reduced by the same tile and merge code as
 // rosen_reduce.  Lattice ensembles are therefore identical, bit for bit, to
 // growing and reducing them alone; real-space ensembles are identical bit for
 // bit when grown alone with the lanes per chain the batch chose (the group
@@ -40,8 +43,20 @@ namespace rosen {
 namespace {
 
 // A member is grown by its own single-ensemble launch from this many waves of
-// resident chains up.
-constexpr int64_t kOwnLaunchWaves = 4;
+// resident chains up.  Where that is the class's own code, four, so that its last
+// wave costs little beside the class kernel's common queue.  Hard spheres and
+// lattice chains with bitmap tables have a faster kernel of their own: one.
+// GB300, batch in the class kernel and by own launches: hard spheres N = 64, k =
+// 32 (19456 chains at once), 8 members of 20000 chains 3.51 -> 2.53 ms, 30000
+// 5.20 -> 3.16, 77000 13.2 -> 6.5, one member of 30000 0.81 -> 0.42; N = 250, k =
+// 64, 4 of 5000 4.41 -> 4.00; lattice N = 512 (24320 at once), 4 of 30000 9.88 ->
+// 3.57, 77000 24.3 -> 7.0; N = 200 (48640), 4 of 77000 2.81 -> 2.84.
+int64_t own_launch_waves(const rosen_ensemble &e)
+{
+    const bool own_kernel = e.model == ROSEN_MODEL_LATTICE ? lattice_has_blocks(e.N)
+                                                           : e.potential != ROSEN_LJ;
+    return own_kernel ? 1 : 4;
+}
 
 struct ClassPlan {
     bool lattice;
@@ -603,7 +618,7 @@ int create(rosen_batch *b, const rosen_ensemble *ens, int n)
                 const rosen_offlattice_params p = off_params(x, 0);
                 res = offlattice_resident_chains(&p);
             }
-            if (res > 0 && x.C >= kOwnLaunchWaves * res) {
+            if (res > 0 && x.C >= own_launch_waves(x) * res) {
                 c.own[m] = 1;
                 if (!c.lattice) {
                     c.own_off[m] = c.own_bytes;

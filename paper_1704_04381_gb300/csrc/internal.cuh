@@ -16,6 +16,8 @@ size_t lattice_smem_bytes(int N, int B);
 // N <= 512); outputs are those of rosen_lattice_grow, bit for bit.
 int lattice_grow_range(const rosen_lattice_params *p, const rosen_lattice_out *o, int64_t c_lo,
                        int64_t c_hi, cudaStream_t s);
+// Whether rosen_lattice_grow grows such chains with bitmap tables.
+bool lattice_has_blocks(int N);
 // Chains the GPU grows at the same time for this ensemble (0 on error).
 int64_t lattice_resident_chains(const rosen_lattice_params *p);
 int lattice_batch_prepare(int B, int Nmax, size_t *smem, int *blocks_per_sm);

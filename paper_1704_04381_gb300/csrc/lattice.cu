@@ -966,7 +966,7 @@ int lattice_grow_range(const rosen_lattice_params *p, const rosen_lattice_out *o
     if (c_hi <= c_lo) return ROSEN_OK;
     LatticeArgs a;
     lattice_make_args(p, o, &a);
-    if (p->N >= kBlocksFromN) return lattice_blocks_launch(a, c_lo, c_hi, s);
+    if (lattice_has_blocks(p->N)) return lattice_blocks_launch(a, c_lo, c_hi, s);
     const int B = lattice_block(p->N);
     if (a.max_att > 1) return lattice_retry_launch(a, p->N, B, c_lo, c_hi, s);
     const size_t smem = lattice_smem_bytes(p->N, B);
@@ -980,9 +980,11 @@ int lattice_grow_range(const rosen_lattice_params *p, const rosen_lattice_out *o
     return check_launch("rosen_lattice_grow");
 }
 
+bool lattice_has_blocks(int N) { return N >= kBlocksFromN; }
+
 int64_t lattice_resident_chains(const rosen_lattice_params *p)
 {
-    if (p->N >= kBlocksFromN) {
+    if (lattice_has_blocks(p->N)) {
         const int64_t warps = blocks_plan(p->N, p->beta_eps != 0.0).resident;
         if (warps < 1) cudaGetLastError();
         return 32 * warps;
