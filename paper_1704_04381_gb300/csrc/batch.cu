@@ -111,7 +111,7 @@ struct rosen_batch {
     unsigned long long *d_counters = nullptr;   // [3], real-space diagnostics
     void *d_rargs = nullptr;              // ReduceArgs[n]
     int64_t *d_tile_off = nullptr;        // [n+1]
-    int64_t total_tiles = 0;
+    int64_t total_tiles = 0, max_tiles = 0;      // of all ensembles, of the largest
     void *d_part = nullptr;
     rosen_stats *d_stats = nullptr;
     cudaStream_t s0 = nullptr;
@@ -407,8 +407,8 @@ int capture(rosen_batch *b)
         note(cudaEventRecord(c.done, c.stream), "record join");
         note(cudaStreamWaitEvent(b->s0, c.done, 0), "join");
     }
-    reduce_batch_launch(b->d_rargs, b->d_tile_off, (int)b->ens.size(), b->total_tiles, b->d_part,
-                        b->d_stats, b->s0);
+    reduce_batch_launch(b->d_rargs, b->d_tile_off, (int)b->ens.size(), b->total_tiles, b->max_tiles,
+                        b->d_part, b->d_stats, b->s0);
     note(cudaGetLastError(), "reduction launch");
     cudaError_t e = cudaStreamEndCapture(b->s0, &g);
     if (first != cudaSuccess) {
@@ -548,6 +548,7 @@ int create(rosen_batch *b, const rosen_ensemble *ens, int n)
         }
         reduce_make_args(&in, rargs.data() + e * reduce_args_size());
         tile_off[e + 1] = tile_off[e] + reduce_tiles(ens[e].C);
+        b->max_tiles = std::max(b->max_tiles, reduce_tiles(ens[e].C));
     }
     b->total_tiles = tile_off[n];
     CK(cudaMalloc(&b->d_rargs, rargs.size()));

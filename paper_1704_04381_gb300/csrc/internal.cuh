@@ -54,10 +54,12 @@ size_t reduce_args_size();
 void reduce_make_args(const rosen_reduce_in *in, void *out);
 int64_t reduce_tiles(int64_t C);
 size_t reduce_partial_bytes();
-// Every tile of every ensemble in one launch, then one block per ensemble
-// merging its partials: the same tile and merge code as rosen_reduce, so the
-// statistics of an ensemble do not depend on the batch it is reduced in.
+// Every tile of every ensemble in one launch, then the merge of each ensemble's
+// partials: the same tile and merge code as rosen_reduce, so the statistics of an
+// ensemble do not depend on the batch it is reduced in.  max_tiles: the most
+// tiles of one ensemble.
 void reduce_batch_launch(const void *dev_args, const int64_t *dev_tile_off, int n_ens,
-                         int64_t total_tiles, void *part, rosen_stats *out, cudaStream_t s);
+                         int64_t total_tiles, int64_t max_tiles, void *part, rosen_stats *out,
+                         cudaStream_t s);
 
 }  // namespace rosen

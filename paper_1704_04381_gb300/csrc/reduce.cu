@@ -298,30 +298,34 @@ __device__ __forceinline__ void reduce_tile(const ReduceArgs &a, int64_t tile, P
     double M = *cluster.map_shared_rank(&block_m, 0);
 #pragma unroll
     for (int r = 1; r < kTileCtas; ++r) M = fmax(M, *cluster.map_shared_rank(&block_m, r));
-    double s[kSums];
+    if (c0 >= a.C) {              // a short tile: no chain in this quarter
+        if (threadIdx.x < kSums) b.v[threadIdx.x] = 0.0;
+    } else {
+        double s[kSums];
 #pragma unroll
-    for (int q = 0; q < kSums; ++q) s[q] = 0.0;
-    uint32_t alive = 0u;
-    if (M > -INFINITY) {
+        for (int q = 0; q < kSums; ++q) s[q] = 0.0;
+        uint32_t alive = 0u;
+        if (M > -INFINITY) {
 #pragma unroll
-        for (int q = 0; q < kPerThread; ++q) {
-            if (lw[q] == -INFINITY) continue;
-            const double w = exp_weight(lw[q] - M, pow2), w2 = w * w;
-            const double u = w2 * A1[q], v = w2 * A2[q];
-            s[0] += w;
-            s[1] += w * A1[q];
-            s[2] += w * A2[q];
-            s[3] += w2;
-            s[4] += u;
-            s[5] += u * A1[q];
-            s[6] += v;
-            s[7] += v * A2[q];
-            ++alive;
+            for (int q = 0; q < kPerThread; ++q) {
+                if (lw[q] == -INFINITY) continue;
+                const double w = exp_weight(lw[q] - M, pow2), w2 = w * w;
+                const double u = w2 * A1[q], v = w2 * A2[q];
+                s[0] += w;
+                s[1] += w * A1[q];
+                s[2] += w * A2[q];
+                s[3] += w2;
+                s[4] += u;
+                s[5] += u * A1[q];
+                s[6] += v;
+                s[7] += v * A2[q];
+                ++alive;
+            }
         }
+        s[8] = (double)alive;
+        s[9] = (double)growths;
+        block_sums(b, s);
     }
-    s[8] = (double)alive;
-    s[9] = (double)growths;
-    block_sums(b, s);
     cluster.sync();
     if (rank == 0 && threadIdx.x < kSums) {
         double t = b.v[threadIdx.x];
@@ -390,9 +394,12 @@ __device__ __forceinline__ void finish_warp(double M, const double *S, int N, in
     }
 }
 
-// Merge the ntiles partials of one ensemble (one cluster): their maximum M,
-// then the sum of every partial's sums scaled by exp(M_t - M) (squared for the
-// sums of w^2).
+// Merge the ntiles partials of one ensemble (one cluster of kCtas blocks): their
+// maximum M, then the sum of every partial's sums scaled by exp(M_t - M) (squared
+// for the sums of w^2).  Partial t belongs to block t / kThreads % kFinalCtas, so
+// that up to kThreads partials one block alone gives the same sums (the others'
+// would be zeros).
+template <int kCtas>
 __device__ __forceinline__ void reduce_final(const Partial *part, int64_t ntiles,
                                              const ReduceArgs &a, rosen_stats *out)
 {
@@ -408,7 +415,7 @@ __device__ __forceinline__ void reduce_final(const Partial *part, int64_t ntiles
     if (threadIdx.x == 0) block_m = M;
     cluster.sync();
 #pragma unroll
-    for (int r = 0; r < kFinalCtas; ++r) M = fmax(M, *cluster.map_shared_rank(&block_m, r));
+    for (int r = 0; r < kCtas; ++r) M = fmax(M, *cluster.map_shared_rank(&block_m, r));
     double s[kSums];
 #pragma unroll
     for (int q = 0; q < kSums; ++q) s[q] = 0.0;
@@ -429,7 +436,7 @@ __device__ __forceinline__ void reduce_final(const Partial *part, int64_t ntiles
     if (rank == 0) {
         if (threadIdx.x < kSums) {
             double t = b.v[threadIdx.x];
-            for (int r = 1; r < kFinalCtas; ++r) t += *cluster.map_shared_rank(&b.v[threadIdx.x], r);
+            for (int r = 1; r < kCtas; ++r) t += *cluster.map_shared_rank(&b.v[threadIdx.x], r);
             b.part[0][threadIdx.x] = t;
         }
         __syncthreads();
@@ -439,10 +446,11 @@ __device__ __forceinline__ void reduce_final(const Partial *part, int64_t ntiles
     cluster.sync();      // (no block leaves while its sums are read)
 }
 
-__global__ void __cluster_dims__(kFinalCtas) __launch_bounds__(kThreads)
+template <int kCtas>
+__global__ void __cluster_dims__(kCtas) __launch_bounds__(kThreads)
     reduce_final_kernel(const Partial *part, int64_t ntiles, const ReduceArgs a, rosen_stats *out)
 {
-    reduce_final(part, ntiles, a, out);
+    reduce_final<kCtas>(part, ntiles, a, out);
 }
 
 // Batched: cluster b reduces global tile b; tile_off[e] .. tile_off[e+1]-1 are
@@ -461,12 +469,13 @@ __global__ void __cluster_dims__(kTileCtas) __launch_bounds__(kThreads)
     reduce_tile(args[lo], b - tile_off[lo], &part[b]);
 }
 
-__global__ void __cluster_dims__(kFinalCtas) __launch_bounds__(kThreads)
+template <int kCtas>
+__global__ void __cluster_dims__(kCtas) __launch_bounds__(kThreads)
     reduce_final_batch_kernel(const Partial *part, const int64_t *tile_off, const ReduceArgs *args,
                               rosen_stats *out)
 {
-    const int e = blockIdx.x / kFinalCtas;
-    reduce_final(part + tile_off[e], tile_off[e + 1] - tile_off[e], args[e], out + e);
+    const int e = blockIdx.x / kCtas;
+    reduce_final<kCtas>(part + tile_off[e], tile_off[e + 1] - tile_off[e], args[e], out + e);
 }
 
 }  // namespace
@@ -499,13 +508,18 @@ void reduce_make_args(const rosen_reduce_in *in, void *out)
 }
 
 void reduce_batch_launch(const void *dev_args, const int64_t *dev_tile_off, int n_ens,
-                         int64_t total_tiles, void *part, rosen_stats *out, cudaStream_t s)
+                         int64_t total_tiles, int64_t max_tiles, void *part, rosen_stats *out,
+                         cudaStream_t s)
 {
     const ReduceArgs *args = reinterpret_cast<const ReduceArgs *>(dev_args);
     Partial *p = reinterpret_cast<Partial *>(part);
     reduce_tiles_batch_kernel<<<(unsigned)(total_tiles * kTileCtas), kThreads, 0, s>>>(
         args, dev_tile_off, n_ens, p);
-    reduce_final_batch_kernel<<<n_ens * kFinalCtas, kThreads, 0, s>>>(p, dev_tile_off, args, out);
+    if (max_tiles <= kThreads)
+        reduce_final_batch_kernel<1><<<n_ens, kThreads, 0, s>>>(p, dev_tile_off, args, out);
+    else
+        reduce_final_batch_kernel<kFinalCtas>
+            <<<n_ens * kFinalCtas, kThreads, 0, s>>>(p, dev_tile_off, args, out);
 }
 
 int reduce_launch(const rosen_reduce_in *in, rosen_stats *out, void *part_ws, cudaStream_t s)
@@ -529,7 +543,10 @@ int reduce_launch(const rosen_reduce_in *in, rosen_stats *out, void *part_ws, cu
     const int64_t tiles = reduce_tiles(in->C);
     Partial *part = reinterpret_cast<Partial *>(part_ws);
     reduce_tiles_kernel<<<(unsigned)(tiles * kTileCtas), kThreads, 0, s>>>(a, part);
-    reduce_final_kernel<<<kFinalCtas, kThreads, 0, s>>>(part, tiles, a, out);
+    if (tiles <= kThreads)
+        reduce_final_kernel<1><<<1, kThreads, 0, s>>>(part, tiles, a, out);
+    else
+        reduce_final_kernel<kFinalCtas><<<kFinalCtas, kThreads, 0, s>>>(part, tiles, a, out);
     return check_launch("rosen_reduce");
 }
 
