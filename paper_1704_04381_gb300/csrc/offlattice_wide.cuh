@@ -409,10 +409,12 @@ __global__ void __launch_bounds__(512, 1) offlattice_wide_kernel(const __grid_co
     float *logm = reinterpret_cast<float *>(smem_raw);
     uint8_t *nth = reinterpret_cast<uint8_t *>(smem_raw + kTable * sizeof(float));
     fill_log_table(logm);
-    for (int q = threadIdx.x; q < kWideSelBytes; q += blockDim.x) {
-        uint32_t v = (uint32_t)q >> 3;
-        for (int t = 0; t < (q & 7); ++t) v &= v - 1u;
-        nth[q] = (uint8_t)(v ? __ffs(v) - 1 : 0);
+    for (int q = threadIdx.x; q < 256; q += blockDim.x) {
+        uint64_t row = 0ull;                 // the set bits of byte q, ascending
+        int shift = 0;
+        for (uint32_t v = (uint32_t)q; v; v &= v - 1u, shift += 8)
+            row |= (uint64_t)(__ffs(v) - 1) << shift;
+        reinterpret_cast<uint64_t *>(nth)[q] = row;
     }
     __syncthreads();
 
@@ -423,7 +425,8 @@ __global__ void __launch_bounds__(512, 1) offlattice_wide_kernel(const __grid_co
                      (size_t)(threadIdx.x / G) * sh.stride;
     float4 *const near = reinterpret_cast<float4 *>(P + 6 * np);   // a near bead per lane
     uint8_t *const tr = reinterpret_cast<uint8_t *>(P + 6 * np + 8 * G);
-    for (int q = g.gl; q < sh.stride; q += G) P[q] = 0.f;   // (what is read is finite)
+    for (int q = g.gl; q < sh.stride / 4; q += G)           // (what is read is finite)
+        reinterpret_cast<float4 *>(P)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncwarp();                         // before restart() writes the same words from other lanes
     const int N = a.N, k = a.k;
     const auto put = [&](int j, float hx, float hy, float hz, float lx, float ly, float lz) {
