@@ -248,18 +248,22 @@ struct WidePlan {
 // Shape for n chains of N beads and k trials whose sums follow gref lanes per
 // chain.  G is the fewest lanes that hold k trials (8 each) and whose scan bits
 // fit a word (N <= 32 G); with few chains it doubles while the warps stay
-// within 9 per SM, where the lanes would idle otherwise and a step's latency
-// counts (N = 64, k = 32, G = 4 / 8 / 16: 2500 chains 0.192 / 0.172 / 0.162
-// ms, 5000 0.210 / 0.186 / 0.243, 10^4 0.264 / 0.270 / 0.342).  A block has
-// the warps that fill an SM's shared memory best, at most 16 (128 registers a
-// thread), fewer where there are not enough chains for every SM.
+// within 9 per SM (k > 16: 12, k > 32: 14, as more trials keep more lanes busy),
+// where the lanes would idle otherwise and a step's latency counts.  G = 4 / 8 /
+// 16 / 32, us: N = 64, k = 32, 700 chains 151 / 123 / 97 / 95, 2000 153 / 125 /
+// 106 / 131, 3500 156 / 133 / 115 / -; k = 64 (8 / 16 / 32), 2000: 162 / 148 /
+// 129; N = 129, k = 64 (8 / 16 / 32), 1500 286 / 222 / 198, 2000 336 / 252 / 226;
+// k = 16, 2000 (8 / 16 / 32) 197 / 187 / 218.  A block has the warps that fill an
+// SM's shared memory best, at most 16 (128 registers a thread), fewer where there
+// are not enough chains for every SM.
 WidePlan wide_plan(const OffArgs &a, int gref, int64_t n, int sms)
 {
     WidePlan w;
     const int N = a.N, k = a.k;
     int G = 4;
     while (8 * G < k || 32 * G < N) G *= 2;
-    while (G < 32 && n * 2 * G <= (int64_t)32 * 9 * sms) G *= 2;
+    const int few = k <= 16 ? 9 : (k <= 32 ? 12 : 14);
+    while (G < 32 && n * 2 * G <= (int64_t)32 * few * sms) G *= 2;
     const int T = ((k + G - 1) / G + 1) / 2 * 2;
     w.fn = nullptr;
 #define ROSEN_WIDE(GG, TT) if (G == GG && T == TT) w.fn = offlattice_wide_kernel<GG, TT>;
