@@ -915,8 +915,9 @@ int lattice_retry_launch(const LatticeArgs &a, int N, int B, int64_t c_lo, int64
     return check_launch("rosen_lattice_grow");
 }
 
-// Chains from this length on grow with bitmap tables (lattice_blocks.cuh),
-// which overtake the scan between N = 128 and 160, athermal and interacting.
+// Chains from this length on may grow with bitmap tables (lattice_blocks.cuh),
+// which overtake the scan between N = 128 and 160, athermal and interacting
+// (which calls do: blocks_win below).
 constexpr int kBlocksFromN = 160;
 
 // Their kernel's shape: blocks of one warp, and the warps the GPU holds at once.
@@ -925,6 +926,7 @@ struct BlocksPlan {
     int entries;
     size_t smem;
     int64_t resident;     // 0: a CUDA error
+    int sms;
 };
 
 BlocksPlan blocks_plan(int N, bool isaw)
@@ -940,16 +942,37 @@ BlocksPlan blocks_plan(int N, bool isaw)
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     b.resident = e == cudaSuccess ? (int64_t)bps * sms : 0;
+    b.sms = e == cudaSuccess ? sms : 0;
     return b;
+}
+
+// Whether n chains of a call grow faster with bitmap tables than by the scan (in
+// blocks of B chains).  In restart mode, where their lanes take the next growth at
+// once (GB300: 1.2 to 2.1 times as fast, 100 to 10^5 chains), and where the scan
+// holds fewer than 256 chains per SM (from N = 209 on: 1.0 to 2.4 times), they do.
+// Below, a round of resident chains takes the two about the same time, the scan
+// 0.9 to 1.1 of the tables', and what counts is how many rounds the call takes
+// either way: N = 180, athermal, us, scan and tables: 30000 chains (1 round each)
+// 160 / 168, 50000 (2, 1) 286 / 189, 70000 (2, 2) 318 / 358, 100000 (3, 2) 475 /
+// 365; beta eps = 0.4: 274 / 255, 477 / 308, 544 / 596, 814 / 615.  Of one round
+// each, the tables except for athermal chains that are stored (the scan's lanes
+// write in step: N = 180, 1000 chains 134 / 155); of three or more, interacting
+// ones (N = 207, 100000 chains 1032 / 957); a single warp's always (N = 200, 1
+// chain 146 / 111).
+bool blocks_win(const BlocksPlan &b, int B, bool isaw, bool restart, bool stored, int64_t n)
+{
+    if (restart || B < 128 || n <= 32) return true;
+    const int64_t scan = (n + 2 * B * (int64_t)b.sms - 1) / (2 * B * (int64_t)b.sms);
+    const int64_t tables = (n + 32 * b.resident - 1) / (32 * b.resident);
+    if (scan != tables) return tables < scan;
+    return isaw ? tables != 2 : tables == 1 && !stored;
 }
 
 // Every warp takes an equal, contiguous share of the chains (at least one per
 // lane), so that all are resident at once.
-int lattice_blocks_launch(const LatticeArgs &a, int64_t c_lo, int64_t c_hi, cudaStream_t s)
+int lattice_blocks_launch(const LatticeArgs &a, const BlocksPlan &b, int64_t c_lo, int64_t c_hi,
+                          cudaStream_t s)
 {
-    const BlocksPlan b = blocks_plan(a.N, a.isaw);
-    if (b.resident < 1)
-        return set_error(ROSEN_ECUDA, "rosen_lattice_grow: %s", cudaGetErrorString(cudaGetLastError()));
     const int64_t n = c_hi - c_lo;
     const int64_t per_warp = std::max<int64_t>(32, (n + b.resident - 1) / b.resident);
     b.kern<<<(unsigned)((n + per_warp - 1) / per_warp), 32, b.smem, s>>>(a, b.entries, per_warp,
@@ -966,8 +989,15 @@ int lattice_grow_range(const rosen_lattice_params *p, const rosen_lattice_out *o
     if (c_hi <= c_lo) return ROSEN_OK;
     LatticeArgs a;
     lattice_make_args(p, o, &a);
-    if (lattice_has_blocks(p->N)) return lattice_blocks_launch(a, c_lo, c_hi, s);
     const int B = lattice_block(p->N);
+    if (lattice_has_blocks(p->N)) {
+        const BlocksPlan b = blocks_plan(a.N, a.isaw);
+        if (b.resident < 1)
+            return set_error(ROSEN_ECUDA, "rosen_lattice_grow: %s",
+                             cudaGetErrorString(cudaGetLastError()));
+        if (blocks_win(b, B, a.isaw, a.max_att > 1, a.trace || a.coords, c_hi - c_lo))
+            return lattice_blocks_launch(a, b, c_lo, c_hi, s);
+    }
     if (a.max_att > 1) return lattice_retry_launch(a, p->N, B, c_lo, c_hi, s);
     const size_t smem = lattice_smem_bytes(p->N, B);
     const int64_t blocks = (c_hi - c_lo + B - 1) / B;
