@@ -586,10 +586,10 @@ __global__ void __launch_bounds__(256) lattice_long_isaw_kernel(const LatticeArg
 // six neighbours are scored as the bitmap kernel for shorter chains does
 // (lattice_blocks.cuh), in 32-bit arithmetic.  Lanes step independently: one
 // whose chain ends takes the next at once instead of waiting for the warp's
-// longest.  Bound by the latency of the probes (L1 and L2 hits).  GB300, 64-bit
-// keys, a site at a time and lanes waiting for one another before, and now: N =
-// 1000, 10^6 chains 21.5 -> 18.8 ms; 4000, 5 10^4: 8.7 -> 6.5; 10^4, 2 10^5:
-// 44 -> 27.  (Interacting chains, with six look-ups a step, lose what they
+// longest (where nothing is stored).  Bound by the latency of the probes (L1 and
+// L2 hits).  GB300, 64-bit keys, a site at a time and lanes waiting for one another
+// before, and now: N = 1000, 10^6 chains 21.5 -> 18.6 ms; 4000, 5 10^4: 8.7 -> 6.4;
+// 10^4, 2 10^5: 44 -> 26.  (Interacting chains, with six look-ups a step, lose what they
 // gain: N = 1000, 2 10^5 chains, beta eps = 0.3, 7.3 ms before, 8.0 this way.)
 constexpr uint32_t kMulXY = 0x9E3779B1u, kMulZ = 0x85EBCA77u;   // hash of (x | y << 16, z)
 
@@ -699,12 +699,11 @@ __device__ __forceinline__ int step_long(LongWalk &w, uint4 *tab, int logH, uint
     return m;
 }
 
-// Outputs of a finished chain (dead: trapped at step i).
-__device__ __forceinline__ void finish_long(const LatticeArgs &a, int64_t c, uint32_t att, int i,
-                                            bool dead, LongWalk &w)
+// Outputs of a finished chain (dead: trapped), but for the rows after a dead end.
+__device__ __forceinline__ void finish_long(const LatticeArgs &a, int64_t c, uint32_t att, bool dead,
+                                            LongWalk &w)
 {
     const int N = a.N;
-    const int64_t C = a.C;
     if (a.attempts) a.attempts[c] = (uint16_t)(att + 1);
     if (dead) w.cnt_lo += 1ull;   // counts[0] = 1 marks the dead end
     if (a.counts)
@@ -723,18 +722,31 @@ __device__ __forceinline__ void finish_long(const LatticeArgs &a, int64_t c, uin
         a.n2rg2[c] = dead ? 0
                           : (int64_t)N * w.sq - ((int64_t)w.sx * w.sx + (int64_t)w.sy * w.sy +
                                                  (int64_t)w.sz * w.sz);
-    if (dead) {
-        if (a.trace) {
-            a.trace[(int64_t)(i - 1) * C + c] = 7u;
-            for (int s = i + 1; s < N; ++s) a.trace[(int64_t)(s - 1) * C + c] = 0xFFu;
+}
+
+// The rows of a trace (7, then 0xFF) and a conformation (zeros) that chains trapped
+// at their step i leave, a chain after another by the whole warp: a lane alone
+// would write up to N rows while 31 others wait (N = 4000, 5000 chains stored, 8.5
+// ms that way, 6.1 by the warp).
+__device__ __forceinline__ void store_tails(const LatticeArgs &a, bool trapped, int64_t c, int i)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    for (unsigned t = __ballot_sync(kAll, trapped); t; t &= t - 1u) {
+        const int from = __ffs(t) - 1, dead = __shfl_sync(kAll, i, from);
+        const int64_t of = __shfl_sync(kAll, c, from);
+        for (int s = dead + (threadIdx.x & 31); s < a.N; s += 32) {
+            if (a.trace) a.trace[(int64_t)(s - 1) * a.C + of] = s == dead ? 7u : 0xFFu;
+            if (a.coords)
+                for (int q = 0; q < 3; ++q) a.coords[((int64_t)s * 3 + q) * a.C + of] = 0;
         }
-        if (a.coords)
-            for (int s = 3 * i; s < 3 * N; ++s) a.coords[(int64_t)s * C + c] = 0;
     }
 }
 
 // Lane l of the grid works in its own table (2^logH entries at ws + l 2^logH)
-// and takes its chains from the counter *next.
+// and takes its chains from the counter *next.  kStore: a trace or conformations
+// are written; then the lanes of a warp start their chains together, so that its
+// stores are contiguous (N = 513, 2 10^5 chains 3.33 -> 3.03 ms).
+template <bool kStore>
 __global__ void __launch_bounds__(256) lattice_long_kernel(const LatticeArgs a, uint4 *ws,
                                                            int64_t lanes, int logH,
                                                            unsigned long long *next)
@@ -753,7 +765,8 @@ __global__ void __launch_bounds__(256) lattice_long_kernel(const LatticeArgs a, 
     int i = 0;
     LongWalk w;
     for (;;) {
-        if (c < 0 && more) {
+        const bool start = !kStore || !__any_sync(0xffffffffu, c >= 0);
+        if (c < 0 && more && start) {
             const unsigned long long n = atomicAdd(next, 1ull);
             more = n < (unsigned long long)a.C;
             if (more) {
@@ -761,24 +774,26 @@ __global__ void __launch_bounds__(256) lattice_long_kernel(const LatticeArgs a, 
                 att = 0u;
                 i = 1;
                 begin_long(w, tab, logH, gen);
-                first_monomer(a, c);
+                if (kStore) first_monomer(a, c);
             }
         }
         if (!__any_sync(0xffffffffu, c >= 0)) break;
+        bool trapped = false;
         if (c >= 0) {
             const uint32_t x = philox(make_uint4(a.chain0 + (uint32_t)c, a.ens,
                                                  (uint32_t)i | (att << 16), 0u), a.key).x;
             int sel = 0;
             const int m = step_long(w, tab, logH, gen, x, seltab, masks, sel);
             if (m > 0) {
-                if (a.trace) a.trace[(int64_t)(i - 1) * a.C + c] = (uint8_t)((m << 3) | sel);
-                if (a.coords) {
+                if (kStore && a.trace)
+                    a.trace[(int64_t)(i - 1) * a.C + c] = (uint8_t)((m << 3) | sel);
+                if (kStore && a.coords) {
                     a.coords[((int64_t)i * 3 + 0) * a.C + c] = w.ex;
                     a.coords[((int64_t)i * 3 + 1) * a.C + c] = w.ey;
                     a.coords[((int64_t)i * 3 + 2) * a.C + c] = w.ez;
                 }
                 if (++i == a.N) {
-                    finish_long(a, c, att, i, false, w);
+                    finish_long(a, c, att, false, w);
                     c = -1;
                 }
             } else if (att + 1 < a.max_att) {
@@ -786,9 +801,14 @@ __global__ void __launch_bounds__(256) lattice_long_kernel(const LatticeArgs a, 
                 i = 1;
                 begin_long(w, tab, logH, gen);
             } else {
-                finish_long(a, c, att, i, true, w);
-                c = -1;
+                finish_long(a, c, att, true, w);
+                if (kStore) trapped = true;
+                else c = -1;
             }
+        }
+        if constexpr (kStore) {
+            store_tails(a, trapped, c, i);
+            if (trapped) c = -1;
         }
         __syncwarp();
     }
@@ -1104,8 +1124,12 @@ extern "C" int rosen_lattice_grow_long(const rosen_lattice_params *p, const rose
     if (a.isaw)
         lattice_long_isaw_kernel<<<grid, 256, 0, s>>>(a, reinterpret_cast<ulonglong2 *>(ws), lanes,
                                                       logH, next);
+    else if (a.trace || a.coords)
+        lattice_long_kernel<true><<<grid, 256, 0, s>>>(a, reinterpret_cast<uint4 *>(ws), lanes, logH,
+                                                       next);
     else
-        lattice_long_kernel<<<grid, 256, 0, s>>>(a, reinterpret_cast<uint4 *>(ws), lanes, logH, next);
+        lattice_long_kernel<false><<<grid, 256, 0, s>>>(a, reinterpret_cast<uint4 *>(ws), lanes, logH,
+                                                        next);
     return check_launch("rosen_lattice_grow_long (kernel launch)");
 }
 
