@@ -40,10 +40,10 @@
 // the same, bit for bit, alone, in any mix, and through the single-ensemble
 // entry points.
 //
-// Device memory of a request (outputs, reduction scratch, the real-space
-// chain counters, a long-chain workspace, stored
-// conformations) comes from one stream-ordered pool and is counted against
-// the budget from admission until it is returned.
+// Device memory of a request (outputs, reduction scratch, the real-space chain
+// counters, a long-chain workspace, stored conformations) comes from one
+// stream-ordered pool and is counted against the budget from admission until it
+// is returned.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -101,7 +101,7 @@ struct Request {
     void *rws = nullptr;       // reduction workspace
     size_t rws_bytes = 0;
     rosen_stats *dstats = nullptr;
-    void *scratch = nullptr;   // real space: two sets of chain counters
+    void *scratch = nullptr;   // real space: two chain counters
     void *long_ws = nullptr;   // long chains: their workspace
     size_t long_bytes = 0;
     cudaStream_t streams[2] = {nullptr, nullptr};   // slices alternate between them
@@ -187,21 +187,28 @@ size_t long_workspace_bytes(const rosen_request &r)
     return align256(std::max(one, std::min(want, kLongWorkspaceCap)));
 }
 
-// Real-space chain counters (one set per stream; shared-memory kernels).  A bit
-// per chain is reserved with them: what a budget or a pool cap admits is a
-// promise to clients and stays what it was when launches shared such a mask.
+// Real-space chain counters (one per stream; shared-memory kernels).
 size_t scratch_bytes(const rosen_request &r)
 {
     if (r.model != ROSEN_MODEL_OFFLATTICE || long_request(r)) return 0;
-    return align256(2 * offlattice_range_counter_bytes() + (size_t)((r.C + 31) / 32) * 4);
+    return align256(2 * offlattice_range_counter_bytes());
 }
 
-// Device bytes a request holds while it runs, and what stored conformations
-// keep after it finishes.
+// Bytes counted beside the counters and not allocated: what a budget admits is a
+// promise to clients and stays what it was when launches shared a bit per chain.
+size_t reserve_bytes(const rosen_request &r)
+{
+    if (r.model != ROSEN_MODEL_OFFLATTICE || long_request(r)) return 0;
+    return align256(2 * offlattice_range_counter_bytes() + (size_t)((r.C + 31) / 32) * 4) -
+           scratch_bytes(r);
+}
+
+// Device bytes a request holds while it runs (reserve_bytes of them are only
+// counted), and what stored conformations keep after it finishes.
 void request_bytes(const rosen_request &r, size_t *work, size_t *coords)
 {
     const size_t C = (size_t)r.C, N = (size_t)r.N;
-    size_t b = long_workspace_bytes(r) + scratch_bytes(r);
+    size_t b = long_workspace_bytes(r) + scratch_bytes(r) + reserve_bytes(r);
     if (r.model == ROSEN_MODEL_LATTICE)
         b += align256(16 * C) + align256(4 * C) + align256(4 * C) + align256(8 * C);
     else
@@ -442,12 +449,11 @@ bool admit(rosen_server *s, Request *q)
     q->ns_per_chain = it != s->rate.end() ? it->second : default_ns_per_chain(q->req);
 
     cudaStream_t s0 = q->streams[0];
-    cudaError_t e = cudaMallocFromPoolAsync(&q->work, q->work_bytes, s->pool, s0);
+    cudaError_t e = cudaMallocFromPoolAsync(&q->work, q->work_bytes - reserve_bytes(q->req), s->pool,
+                                            s0);
     if (e == cudaSuccess && q->coord_bytes)
         e = cudaMallocFromPoolAsync(&q->coords, q->coord_bytes, s->pool, s0);
-    if (e == cudaSuccess) {
-        carve(q);
-    }
+    if (e == cudaSuccess) carve(q);
     // The second stream starts after the allocation and the set-up.
     if (e == cudaSuccess) e = cudaEventRecord(q->join, s0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(q->streams[1], q->join, 0);
