@@ -227,16 +227,21 @@ uint64_t rate_key(const rosen_request &r)
            ((uint64_t)(r.k & 0xFFFF) << 32) | (uint64_t)(r.N / 16);
 }
 
-// First estimate of a class's GPU time per chain (ns), from GB300 timings of
-// the single-ensemble kernels at N = 64 (lattice 1.2 ns, hard spheres 0.55 k,
-// Lennard-Jones 1.8 k per chain) scaled by N^2; refined by measured slices.
+// First estimate of a class's GPU time per chain (ns), fitted to GB300 timings of
+// the single-ensemble kernels (trials grow with N and the scan with N^2); refined
+// by measured slices.  Measured and estimated: athermal lattice N = 16 / 64 / 200 /
+// 512 0.09 / 0.55 / 4.4 / 19.7 and 0.10 / 0.60 / 3.9 / 18.9 (interacting 0.14 /
+// 0.92 / 7.2 / 30.7); hard spheres k = 32, N = 64 / 256 / 1000 9.1 / 91 / 994 and
+// 9.6 / 80 / 949, N = 512, k = 8 / 128 148 / 465 and 236 / 419; Lennard-Jones k =
+// 32, N = 16 / 64 / 256 8.1 / 49 / 406 and 8.8 / 57 / 460, N = 64, k = 8 / 128 31 /
+// 192 and 25 / 181.
 double default_ns_per_chain(const rosen_request &r)
 {
-    const double f = ((double)r.N / 64.0) * ((double)r.N / 64.0);
-    double base;
-    if (r.model == ROSEN_MODEL_LATTICE) base = 1.2;
-    else base = (r.potential == ROSEN_LJ ? 1.8 : 0.55) * (double)r.k;
-    return std::max(0.05, base * f);
+    const double n = (double)r.N / 64.0, k = (double)r.k;
+    if (r.model == ROSEN_MODEL_LATTICE)
+        return 0.05 + (r.beta_eps == 0.0 ? 0.55 : 0.9) * pow(n, 1.7);
+    return r.potential == ROSEN_LJ ? 1.3 * k * pow(n, 1.2) + 15.0 * n * n
+                                   : 0.19 * k * n + 3.5 * n * n;
 }
 
 int validate_request(const rosen_request &r)
