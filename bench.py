@@ -66,6 +66,20 @@ def brute_offlattice_ops(N, k):
     return BRUTE_OFF_PAIR * k * (N - 1) * (N - 2) // 2 + BRUTE_OFF_TRIAL * k * (N - 1)
 
 
+def wide_kernel_name(N, k, C, dev):
+    """The hard-sphere kernel's shape for C chains: G lanes per chain, T trials per
+    lane (the rule of wide_plan in csrc/offlattice.cu)."""
+    import torch
+    G = 4
+    while 8 * G < k or 32 * G < N:
+        G *= 2
+    warps = (9 if k <= 16 else 12 if k <= 32 else 14) \
+        * torch.cuda.get_device_properties(dev).multi_processor_count
+    while G < 32 and C * 2 * G <= 32 * warps:
+        G *= 2
+    return "offlattice_wide_kernel<%d,%d>" % (G, ((k + G - 1) // G + 1) // 2 * 2)
+
+
 # Work the kernels actually execute, in 32-bit lane operations (they test only
 # the monomers that can reach a trial):
 #  lattice: 6 per pair test (add, range test, gather multiply, shift, table
@@ -303,7 +317,7 @@ def run_ours(args):
             sops = brute_offlattice_ops(N, K_TRIALS) * C
             part.update({"fp64_redecided_steps": cnt[0] / reps,
                          "listed_beads_per_step": listed / (C * (N - 1))})
-            kname = ("offlattice_wide_kernel<4,8>"
+            kname = (wide_kernel_name(N, K_TRIALS, C, dev)
                      if REAL_POT == "hard_sphere"
                      else "offlattice_queue_kernel<LJ, k=%d, beta eps %g>" % (K_TRIALS, REAL_BETA))
         part["ops_per_chain"] = ops / C

@@ -280,8 +280,9 @@ __global__ void __launch_bounds__(256) lattice_retry_kernel(const LatticeArgs a,
 
 // Persistent batch kernel: blocks take (ensemble, chain range) items from a
 // queue (items sorted by decreasing cost) until it is empty; every chain is
-// grown by the same lattice_chain code as in the single-ensemble kernel, so
-// its results do not depend on the batch it is grown in.
+// grown by lattice_chain, the scan of lattice_lane_kernel, at any N (the bitmap
+// tables of longer chains give the same outputs bit for bit), so its results do
+// not depend on the batch it is grown in.
 __global__ void __launch_bounds__(256) lattice_batch_kernel(const LatticeArgs *__restrict__ ens,
                                                             const BatchItem *__restrict__ items,
                                                             int n_items, int *head)

@@ -21,12 +21,13 @@
 // its lane alone with the whole warp's table, once the other lanes are done:
 // 32 times the entries, more than the blocks of any chain.
 //
-// Bound by latency: 5 warps per SM at N = 512 (9 at 256), 470 instructions a
-// step, issue 34%.  GB300, scan kernel and now: athermal N = 160, 4 10^5 chains
+// Bound by latency: 5 warps per SM at N = 512 (9 at 256), 454 instructions a
+// step, issue 33%.  GB300, scan kernel and now: athermal N = 160, 4 10^5 chains
 // 1.32 -> 1.12 ms; 224, 2 10^5: 1.56 -> 1.10; 300, 10^5: 1.80 -> 0.81; 512, 5
 // 10^5: 26.5 -> 9.7; beta eps = 0.4, N = 160, 3 10^5: 1.75 -> 1.64; 224, 2
 // 10^5: 2.69 -> 1.95; 512, 2 10^5: 18.4 -> 7.2.  At N = 128 the scan is faster
-// (1.02 against 1.21 ms; 1.08 against 1.35 interacting).  Tried and not kept:
+// (1.02 against 1.21 ms; 1.08 against 1.35 interacting); between 160 and 208 it
+// depends on the call (blocks_win in lattice.cu).  Tried and not kept:
 // buckets of four tags in one load (10.7 ms at N = 512), two buckets per block
 // without a loop (overflows: 36 ms).
 #pragma once

@@ -94,8 +94,9 @@ __global__ void __launch_bounds__(256, 4) offlattice_queue_kernel(const OffArgs 
 // decreasing cost; ticket t of a counter is chain t % chains_per_block of
 // item t / chains_per_block.  Every group takes its own tickets, keeps the
 // arguments of its current ensemble in shared memory, and grows each chain
-// with the same off_chain code as the single-ensemble kernels -- no group
-// waits for the others of its block.
+// with off_chain -- the code of the single-ensemble Lennard-Jones kernels; hard
+// spheres alone grow with offlattice_wide_kernel, whose outputs equal off_chain's
+// bit for bit.  No group waits for the others of its block.
 template <int G, int T, bool LJ>
 __global__ void __launch_bounds__(256, 4) offlattice_batch_kernel(const OffArgs *__restrict__ ens,
                                                                   const BatchItem *__restrict__ items,
@@ -417,15 +418,16 @@ int offlattice_validate(const rosen_offlattice_params *p, const rosen_offlattice
     return ROSEN_OK;
 }
 
-// Default lanes per chain for the shared-memory kernels (measured on GB300):
-// at N = 64 hard spheres run best with two chains per warp (16 lanes) and
-// Lennard-Jones -- whose pair work is several times heavier -- with a whole
-// warp per chain once k > 16.  Longer chains spend more of each step in the
-// scan of earlier beads, which a whole warp does twice as fast: from N = 100
-// every k takes 32 lanes (N = 128 / 256, hard spheres k = 32: 11.4 / 17.2 ms
-// with 32 lanes against 13.7 / 38.0 ms with 16; LJ k = 16: 25.9 / 46.0
-// against 29.3 / 71.8 ms).  N = 0: the chain length is not known (the
-// long-chain kernel, whose near lists come from cells).
+// Default lanes per chain of off_chain with shared memory (measured on GB300).
+// Lennard-Jones at N = 64 runs best with a whole warp per chain once k > 16, with
+// 16 lanes below.  Longer chains spend more of each step in the scan of earlier
+// beads, which a whole warp does twice as fast: from N = 100 every k takes 32
+// lanes (k = 16, N = 128 / 256: 25.9 / 46.0 ms with 32 lanes against 29.3 / 71.8
+// with 16, a bead at a time).  For hard spheres in rosen_offlattice_grow the value
+// is only the order of the R_g^2 sum (wide_plan picks the lanes); in a batch's
+// class kernel it is the shape before tuning (N = 64, k = 32, 16 lanes: two chains
+// per warp).  N = 0: the chain length is not known (the long-chain kernel, whose
+// near lists come from cells).
 int offlattice_default_lanes(int k, bool lj, int N)
 {
     if (N >= 100) return 32;

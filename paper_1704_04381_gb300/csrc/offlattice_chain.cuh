@@ -928,7 +928,7 @@ __device__ __forceinline__ void off_chain(const OffArgs &a, int64_t c, const W &
                 }
             } else {
                 // Two beads per instruction; a bead beyond the cutoff adds zeros
-                // (instead of a branch per bead).  Issue-bound; of 935 warp
+                // (instead of a branch per bead).  Issue-bound; of 881 warp
                 // instructions per chain step (N = 64, k = 32) the pairs take
                 // a quarter and their error bounds a sixth.  GB300, a bead at a
                 // time before: k = 16 / 32 / 64, 5 10^5, 5 10^5, 3 10^5 chains

@@ -33,9 +33,11 @@
 // 32: N = 64, 10^7 chains 171 -> 91 ms; N = 128, 2 10^5: 11.3 -> 5.8; N = 256,
 // 6 10^4: 10.4 -> 5.5; N = 512, 2 10^4: 17.7 -> 6.3; N = 1024, 5 10^3: 18.5 ->
 // 5.4.  N = 64: k = 16, 5 10^5 chains 7.9 -> 3.7; k = 64, 3 10^5: 8.3 -> 5.0;
-// k = 128, 2 10^5: 9.6 -> 6.2; k = 32, 100 chains 0.23 -> 0.12.  Tried and not kept: all trials
-// through dir32x2 (13.5 ms), per-chain lists ranked by votes (12.5), the next
-// step's trials drawn beside the selection (11.4: more registers moved).
+// k = 128, 2 10^5: 9.6 -> 6.2; k = 32, 100 chains 0.19 -> 0.08.  (One or two trials
+// of N > 128, too few for any lanes to share, take 4 to 9 us longer: k = 2, N = 200,
+// 2000 chains 77 -> 84 us.)  Tried and not kept: all trials through dir32x2 (13.5
+// ms), per-chain lists ranked by votes (12.5), the next step's trials drawn beside
+// the selection (11.4: more registers moved).
 #pragma once
 
 #include "offlattice_chain.cuh"
