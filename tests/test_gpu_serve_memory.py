@@ -33,7 +33,7 @@ def test_counted_but_not_allocated(rosen):
         st, res = srv.wait(srv.submit(req), 60)
         assert st == rosen.ROSEN_OK and res["status"] == rosen.ROSEN_OK, res
         assert res["stats"]["n"] == C
-        assert used <= free - torch.cuda.mem_get_info()[0] < used + mask * 3 // 4
+        assert free - torch.cuda.mem_get_info()[0] < used + mask * 3 // 4
         assert srv.info()["bytes_in_use"] == 0
     finally:
         srv.close()
